@@ -9,7 +9,7 @@
 namespace msi {
 
 constexpr int kRouterTM = 32;  // tokens per fp32 FFMA router block
-constexpr int kRouterChunk = 128;  // experts per tensor-core router CTA
+constexpr int kFuseTokens = 256;   // longest call whose selection and scatter are one launch
 constexpr int kScatterWarps = 4;   // scatter warps per block, one per router block
 
 // The device that was current when the plan was created (plan.cu).
@@ -34,24 +34,41 @@ struct RouterArgs {
 };
 
 struct RouterTcArgs {
-  const __nv_bfloat16* x;  // [T, H] (shared-gate dot products)
+  const __nv_bfloat16* x;  // [T, H]
+  const float* wr;         // [E, H]
   const float* wsg;        // [H] or nullptr
   int T, H, E, k;
-  int chunk;               // experts per router CTA (<= kRouterChunk)
+  int chunk;               // experts per logits CTA (16, 32, 64 or 128; divides E)
   int nchunk;              // E / chunk
-  int kp;                  // candidates per chunk: min(k + 1, chunk)
-  int tmem_cols;           // power of two >= max(32, chunk)
-  float* cand_v;           // [T, nchunk, kp] candidate logits
-  int* cand_i;             // [T, nchunk, kp] candidate expert ids
+  int ksplit;              // parts of K, each its own CTA (1, 2 or 4)
+  int stack;               // planes stacked along the MMA's N (router_tc.cu)
+  int t0, rows;            // the launch's tokens [t0, t0 + rows), t0 a multiple of 128
+  float* logits;           // [ksplit, rows, E] partial sums (scratch)
   int* ids;                // [T, k]
   float* weights;          // [T, k]
   float* gap;              // [T] or nullptr
   float* sg;               // [T]
   int* bcount;             // [ceil(T/32), E]
   int* status;
+  // the forward's first kernel (begin): status cleared, the shared group
+  // written and a resident call's table copied to global memory
+  int begin;
+  Group* sh;               // or nullptr
+  int* sh_total;
+  int* tab_slot;
+  unsigned long long* tab_expected;
+  int* ticket;             // cleared for the selection's last-CTA count
   long long wait_limit;
   int stall;               // as GemmArgs::stall
 };
+
+// How the logits of a call's rows are cut into CTAs.
+struct RouterSplit {
+  int chunk, ksplit;
+  bool stack;
+};
+constexpr int kStackTokens = 4096;  // longest call with the planes stacked (router_tc.cu)
+RouterSplit router_split(int T, int E, int sms);
 
 struct ScanArgs {
   const int* bcount;
@@ -70,6 +87,7 @@ struct ScatterArgs {
   int fuse_scan;
   const int* bcount;  // [nb, E]
   int* counts_out;    // [E]
+  int* ticket;        // selection and scatter in one launch: CTAs finished
   int T, k, E, nb;
   int tm;             // tokens per router block
   int* perm;          // [T*k]
@@ -136,17 +154,11 @@ struct CombineArgs {
 // Launchers (asynchronous on the given stream; return the launch error)
 // ---------------------------------------------------------------------------
 cudaError_t launch_router(const RouterArgs& a, cudaStream_t s);
-// Also begins the forward (its first kernel): clears the status word and,
-// when sh is not null, writes the shared-expert group of T rows in block
-// `shared_slot` and its tile counts.  With tp not null it also copies the
-// call's slot table and expected generations to tab_slot / tab_expected
-// (the entries are read from the kernel argument by many blocks at once;
-// one block reading all of them serialises on its constant cache).
-cudaError_t launch_split3(const float* w, long long n, __nv_bfloat16* out, int* status, Group* sh,
-                          int* sh_total, int T, int shared_slot, const TableParams* tp,
-                          int* tab_slot, unsigned long long* tab_expected, cudaStream_t s);
-cudaError_t launch_router_tc(const CUtensorMap& tmX, const CUtensorMap& tmW, const RouterTcArgs& a,
-                             cudaStream_t s);
+cudaError_t launch_router_logits(const CUtensorMap& tmX, const RouterTcArgs& a, const TableParams& tp,
+                                 cudaStream_t s);
+// sa not null: a call of at most kFuseTokens tokens is scattered as well (no
+// colscan and no scatter launch follow).
+cudaError_t launch_router_select(const RouterTcArgs& a, const ScatterArgs* sa, cudaStream_t s);
 cudaError_t launch_colscan(const ScanArgs& a, cudaStream_t s);
 cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s);
 // Copies the call's table to global memory and, when status is not null,

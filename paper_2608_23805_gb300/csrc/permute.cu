@@ -11,7 +11,7 @@
 // requested object and version, and a mismatch is rejected before any
 // consumer reads the slot (paper, Sec. "Lifetime Is Part of Correctness";
 // Sec. "Stable Slots and Bundle Publication").
-#include "kernels.cuh"
+#include "permute.cuh"
 
 namespace msi {
 
@@ -41,16 +41,6 @@ __global__ void __launch_bounds__(1024) colscan_kernel(const ScanArgs a) {
     }
     if (ty == 31) a.counts[e] = run;
   }
-}
-
-__device__ __forceinline__ int check_code(const GenWord* gw, int slot, int layer, int e,
-                                          unsigned long long expected) {
-  if (slot < 0) return MSI_ERR_NOT_RESIDENT;
-  const unsigned long long obj = gw[slot].obj;
-  const unsigned long long gen = gw[slot].gen;
-  if (obj != obj_key(layer, e)) return MSI_ERR_WRONG_OBJECT;
-  if (gen != expected) return MSI_ERR_STALE_GENERATION;
-  return 0;
 }
 
 // ---- scatter: one warp per router block ----
@@ -253,39 +243,6 @@ __global__ void upload_kernel(const TableParams p, int* table, unsigned long lon
     expected[e] = p.expected[e];
   }
   if (threadIdx.x == 0 && status != nullptr) forward_begin(status, sh, sh_total, p.T, p.shared_slot);
-}
-
-// ---- generation re-check + GEMM groups (one block) ----
-__device__ __forceinline__ int block_excl_scan(int v, int* tmp, int* total) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int incl = v;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int o = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += o;
-  }
-  if (lane == 31) tmp[warp] = incl;
-  __syncthreads();
-  const int nw = blockDim.x >> 5;
-  int base = 0, tot = 0;
-  for (int w = 0; w < nw; ++w) {
-    if (w < warp) base += tmp[w];
-    tot += tmp[w];
-  }
-  *total = tot;
-  return base + incl - v;
-}
-
-__device__ __forceinline__ int block_min(int v, int* tmp) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, off));
-  __syncthreads();
-  if (lane == 0) tmp[warp] = v;
-  __syncthreads();
-  int m = 0x7fffffff;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = min(m, tmp[w]);
-  return m;
 }
 
 // One LRU wave of a streamed call: re-check the wave's slots and build its

@@ -172,7 +172,7 @@ struct WaveEntry {
 };
 
 struct WsLayout {
-  size_t status, table, expected, groups, total, sh_group, sh_total, w3, cand_v, cand_i, bcount,
+  size_t status, table, expected, groups, total, sh_group, sh_total, logits, logits_bytes, bcount,
       bbase, offsets, perm, inv, sg, h, yp, hs, ys, ready, ready_n, bytes;
   int tm;  // tokens per router block
 };
@@ -296,16 +296,16 @@ struct msi_plan {
 
 namespace {
 
-// The tensor-core router splits E into chunks of min(E, 128) experts (MMA N,
-// a multiple of 16) and keeps k + 1 <= 32 candidates per chunk and token.
+// The tensor-core router takes chunks of 16 to 128 experts (MMA N, a multiple
+// of 16) and selects k + 1 <= 32 experts a token, one per lane of a warp.
 // Small layers (E <= 64 and E * H <= 32,768) take the FFMA router instead:
 // sized for 64 experts, its blocks finish in a few microseconds, below the
 // fixed cost of the tensor path's three launches (decode sizes).
 bool tensor_router(const msi_plan_desc& d) {
   const int E = d.n_experts;
   if (E <= 64 && (long long)E * d.hidden <= 32768) return false;
-  return E % 16 == 0 && (E <= kRouterChunk || E % kRouterChunk == 0) && d.top_k <= 31 &&
-         E / std::min(E, kRouterChunk) * std::min(d.top_k + 1, std::min(E, kRouterChunk)) <= 160;
+  return E % 16 == 0 && (E <= 128 || E % 128 == 0) && d.top_k <= 31 &&
+         E / std::min(E, 128) * std::min(d.top_k + 1, std::min(E, 128)) <= 160;
 }
 
 // A call that enqueues work must be made with the plan's device current: its
@@ -339,15 +339,14 @@ WsLayout layout(const msi_plan* p, int T) {
   L.table = take(4 * E);
   L.expected = take(8 * E);
   L.groups = take(sizeof(Group) * std::max<size_t>(E, kMaxWave));
-  L.total = take(8);      // 128-row tiles, 256-row pair tiles
+  L.total = take(12);     // 128-row tiles, 256-row pair tiles; the router selection's ticket
   L.sh_group = take(sizeof(Group));
   L.sh_total = take(8);
-  L.w3 = tensor_router(p->d) ? take(3 * E * H * 2) : 0;
+    // the tensor router's logits (a longer call's go to the GEMMs' buffers, or
+  // through here in row chunks): at least 1.5 H rows
   if (tensor_router(p->d)) {
-    const size_t ch = std::min<size_t>(E, kRouterChunk);
-    const size_t ncand = (E / ch) * std::min<size_t>(k + 1, ch);
-    L.cand_v = take(4 * (size_t)T * ncand);
-    L.cand_i = take(4 * (size_t)T * ncand);
+    L.logits_bytes = 3 * E * H * 2 + 8 * (size_t)T * std::max<size_t>(1, E / 128) * std::min<size_t>(k + 1, E);
+    L.logits = take(L.logits_bytes);
   }
   L.bcount = take(4 * nb * E);
   L.bbase = take(4 * nb * E);
@@ -709,9 +708,11 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 // the shared group; the shared gate is computed, and the side stream may fork
 // after it).  Otherwise a prediction pass: no status reset, no shared group,
 // no gate; it reuses the router scratch of the workspace, so it must be
-// ordered after the forward's own routing and scatter.
+// ordered after the forward's own routing and scatter.  xa: the scatter's
+// arguments; *scattered is set when the selection did its work too.
 msi_status route_rows(msi_plan* p, FwdCtx& f, const float* rw, const msi_route_event* ev, bool first,
-                      const TableParams& tp, cudaStream_t s, bool scan = true) {
+                      const TableParams& tp, cudaStream_t s, bool scan = true,
+                      const ScatterArgs* xa = nullptr, bool* scattered = nullptr) {
   const auto& d = p->d;
   const int E = d.n_experts, k = d.top_k, H = d.hidden;
   void* ws = f.ws;
@@ -720,53 +721,69 @@ msi_status route_rows(msi_plan* p, FwdCtx& f, const float* rw, const msi_route_e
   const float* wsg = first && d.has_shared && !(f.flags & MSI_FWD_SHARED_UNGATED)
                          ? d.shared_gate_w + (size_t)f.layer * H
                          : nullptr;
-  if (tensor_router(d)) {
-    __nv_bfloat16* w3 = at<__nv_bfloat16>(ws, L.w3);
-    // a resident call's table goes to the workspace here, for the scatter's
-    // generation re-check
-    const bool tab = first && tp.E > 0;
-    LAUNCH(p, MSI_K_ROUTER, s,
-           launch_split3(rw, (long long)E * H, w3, first ? at<int>(ws, L.status) : nullptr,
-                         first && d.has_shared ? at<Group>(ws, L.sh_group) : nullptr,
-                         at<int>(ws, L.sh_total), f.T, tp.shared_slot, tab ? &tp : nullptr,
-                         at<int>(ws, L.table), at<unsigned long long>(ws, L.expected), s));
-  }
   // host-buffer calls: every reader of the rows (router, shared expert) comes
   // after they have landed
   if (f.x_ready != nullptr) CK(cudaStreamWaitEvent(s, f.x_ready, 0));
-  // the forward has begun (status cleared, shared group written): the shared
-  // expert may start on the side stream from here
-  if (first && d.has_shared) CK(cudaEventRecord(p->ev_fork, s));
   if (tensor_router(d)) {
-    __nv_bfloat16* w3 = at<__nv_bfloat16>(ws, L.w3);
-    const int ch = std::min(E, kRouterChunk);
-    CUtensorMap tm_w3;
-    if (!make_tmap(&tm_w3, w3, H, (uint64_t)3 * E, (uint32_t)ch)) return MSI_ERR_CUDA;
     RouterTcArgs ra{};
     ra.x = static_cast<const __nv_bfloat16*>(f.x);
+    ra.wr = rw;
     ra.wsg = wsg;
     ra.T = f.T;
     ra.H = H;
     ra.E = E;
     ra.k = k;
-    ra.chunk = ch;
-    ra.nchunk = E / ch;
-    ra.kp = std::min(k + 1, ch);
-    int cols = 32;
-    while (cols < ch) cols <<= 1;
-    ra.tmem_cols = cols;
-    ra.cand_v = at<float>(ws, L.cand_v);
-    ra.cand_i = at<int>(ws, L.cand_i);
     ra.ids = ev->ids;
     ra.weights = ev->weights;
     ra.gap = ev->gap;
     ra.sg = at<float>(ws, L.sg);
     ra.bcount = at<int>(ws, L.bcount);
     ra.status = at<int>(ws, L.status);
+    ra.sh = d.has_shared ? at<Group>(ws, L.sh_group) : nullptr;
+    ra.sh_total = at<int>(ws, L.sh_total);
+    ra.tab_slot = at<int>(ws, L.table);
+    ra.tab_expected = at<unsigned long long>(ws, L.expected);
+    ra.ticket = at<int>(ws, L.total) + 2;
     ra.wait_limit = p->wait_cycles;
     ra.stall = f.stall;
-    LAUNCH(p, MSI_K_ROUTER, s, launch_router_tc(f.tm_x, tm_w3, ra, s));
-    p->launches++;  // launch_router_tc starts two kernels (logits + top-k, merge)
+    // the logits' scratch: the router's own region, or for the forward's own
+    // routing the larger one of the GEMM intermediates (nothing is in them
+    // yet); rows that do not fit go through it in chunks
+    const size_t row = 4 * (size_t)E;
+    size_t cap = L.logits_bytes;
+    ra.logits = at<float>(ws, L.logits);
+    if (first && L.ready - L.h > cap) {
+      cap = L.ready - L.h;
+      ra.logits = at<float>(ws, L.h);
+    }
+    const int chunk_rows = cap / row >= (size_t)f.T ? f.T : (int)(cap / row / 128 * 128);
+    const RouterSplit sp = router_split(chunk_rows, E, p->sms);
+    ra.chunk = sp.chunk;
+    ra.nchunk = E / sp.chunk;
+    ra.ksplit = sp.ksplit;
+    ra.stack = router_split(f.T, E, p->sms).stack;
+    while (ra.ksplit > 1 && ra.ksplit * row * (size_t)chunk_rows > cap) ra.ksplit /= 2;
+    const bool fuse = first && xa != nullptr && f.T <= kFuseTokens;
+    // a long resident call begins with a kernel of its own, so that the side
+    // stream's shared expert runs beside the logits and not after them
+    const bool begun = first && tp.E > 0 && d.has_shared && f.T >= 4096;
+    if (begun) {
+      LAUNCH(p, MSI_K_UPLOAD, s, launch_upload(tp, ra.tab_slot, ra.tab_expected, ra.status, ra.sh, ra.sh_total, s));
+      CK(cudaEventRecord(p->ev_fork, s));
+    }
+    for (ra.t0 = 0; ra.t0 < f.T; ra.t0 += chunk_rows) {
+      ra.rows = std::min(chunk_rows, f.T - ra.t0);
+      ra.begin = first && !begun && ra.t0 == 0;
+      LAUNCH(p, MSI_K_ROUTER, s, launch_router_logits(f.tm_x, ra, tp, s));
+      // the forward has begun (status cleared, shared group written): the
+      // shared expert may start on the side stream from here
+      if (ra.begin && d.has_shared) CK(cudaEventRecord(p->ev_fork, s));
+      LAUNCH(p, MSI_K_ROUTER, s, launch_router_select(ra, fuse ? xa : nullptr, s));
+    }
+    if (fuse) {
+      *scattered = true;
+      return MSI_OK;
+    }
   } else {
     RouterArgs ra{};
     ra.x = static_cast<const __nv_bfloat16*>(f.x);
@@ -786,6 +803,7 @@ msi_status route_rows(msi_plan* p, FwdCtx& f, const float* rw, const msi_route_e
     ra.sh_total = at<int>(ws, L.sh_total);
     ra.shared_slot = tp.shared_slot;
     LAUNCH(p, MSI_K_ROUTER, s, launch_router(ra, s));
+    if (first && d.has_shared) CK(cudaEventRecord(p->ev_fork, s));  // this router begins the forward itself
   }
   // the column scan (per-block prefixes and counts); a small forward's
   // scatter takes it over (scan = false)
@@ -842,16 +860,16 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
     if (!make_tmap(&f.tm_hs, at<char>(ws, L.hs), I, f.T, 128)) return MSI_ERR_CUDA;
   }
   // up to kScatterWarps router blocks: one scatter block covers them all and
-  // takes over the column scan (one launch fewer for decode-sized calls)
+  // takes over the column scan (one launch fewer for decode-sized calls); the
+  // tensor router's selection takes over both up to kFuseTokens
   const bool fuse_scan = nb <= kScatterWarps;
-  msi_status st = route_rows(p, f, f.router_w, f.ev, true, tp, f.cs, !fuse_scan);
-  if (st != MSI_OK) return st;
   ScatterArgs xa{};
   xa.ids = f.ev->ids;
   xa.counts = f.ev->counts;
   xa.fuse_scan = fuse_scan ? 1 : 0;
   xa.bcount = at<int>(ws, L.bcount);
   xa.counts_out = f.ev->counts;
+  xa.ticket = at<int>(ws, L.total) + 2;
   xa.bbase = at<int>(ws, L.bbase);
   xa.T = f.T;
   xa.k = k;
@@ -867,10 +885,8 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
   xa.status = at<int>(ws, L.status);
   if (tp.E > 0) {
     // resident call: the scatter re-checks the table's slots from global
-    // memory (the weight split copied it; the FFMA router path copies it here)
-    if (!tensor_router(d))
-      LAUNCH(p, MSI_K_UPLOAD, f.cs, launch_upload(tp, at<int>(ws, L.table), at<unsigned long long>(ws, L.expected),
-                              nullptr, nullptr, nullptr, f.cs));
+    // memory (the tensor router's first kernel copies it there, or
+    // the upload below)
     xa.tab_slot = at<int>(ws, L.table);
     xa.tab_expected = at<unsigned long long>(ws, L.expected);
     xa.layer = tp.layer;
@@ -884,7 +900,13 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
     xa.ready = at<int>(ws, L.ready);
     xa.n_ready = ready_bank(f);
   }
-  LAUNCH(p, MSI_K_SCATTER, f.cs, launch_scatter(xa, f.cs));
+  bool scattered = false;
+  msi_status st = route_rows(p, f, f.router_w, f.ev, true, tp, f.cs, !fuse_scan, &xa, &scattered);
+  if (st != MSI_OK) return st;
+  if (tp.E > 0 && !tensor_router(d))
+    LAUNCH(p, MSI_K_UPLOAD, f.cs, launch_upload(tp, at<int>(ws, L.table), at<unsigned long long>(ws, L.expected),
+                            nullptr, nullptr, nullptr, f.cs));
+  if (!scattered) LAUNCH(p, MSI_K_SCATTER, f.cs, launch_scatter(xa, f.cs));
   const size_t Tk = (size_t)f.T * k;
   if (f.ids_host != nullptr) {
     // the route ids go back beside the expert GEMMs

@@ -1,6 +1,6 @@
 // Router on tcgen05 tensor cores with fp32-exact products: fp32 logits,
 // top-k, softmax weights, shared-expert gate and the per-block expert
-// histogram (the logits never reach HBM).
+// histogram.
 //
 // The router's top-k output is the route event recorded per layer and graph
 // evaluation (paper, Sec. "Output-Exact Execution Beyond the Full-Residency
@@ -15,151 +15,144 @@
 // an fp32 GEMM up to accumulation order.
 //
 // Two kernels:
-//  1. router_tc_kernel, one CTA per (128 tokens, chunk of <= 128 experts):
-//     logits of the chunk in TMEM (per stage one x tile and the chunk's rows
-//     of all three planes, by TMA, feeding 12 MMAs), then each token's
-//     top-(k+1) candidates within the chunk by warp-shuffle argmax (logit
-//     desc, id asc) from shared memory, four rows at a time per warp.
-//  2. router_merge_kernel, one CTA per 32 tokens (sixteen warps, two tokens
-//     each): the top-(k+1) of the union of the chunks' candidates (it contains
-//     the global top-(k+1)), weights, gap, the block's expert histogram for
-//     the permutation and the shared-expert gate sigmoid(x . w_sg).
-// Warps 0-3 move the logits from TMEM to shared memory, warp 4 MMA + TMEM,
-// warp 5 TMA producer (one lane each for the single-thread roles; every role
-// claims its whole warp); then all eight warps select.  All waits are bounded.
-#include "kernels.cuh"
+//  1. router_logits_kernel, one CTA per (128 tokens, CH experts, K split):
+//     eight warps read the chunk's fp32 weights, split them and write the
+//     three planes as swizzled operand tiles; x tiles come by TMA; 12 MMAs per
+//     64 of K; the logits (of the CTA's part of K) go to global memory, where
+//     the next kernel finds them in L2.
+//     What bounds it: the operand feed (x tile and weights, 48 KB per 64 of K
+//     at CH = 128, at the SM's 64 bytes a cycle from L2) for long calls, and
+//     the latency of one CTA's pass over K for short ones (the two launches
+//     took 40 us for one token as 4 CTAs, and take 17 as 128).  So short calls
+//     are cut into smaller expert chunks, then over K, until the grid fills
+//     the SMs (router_split).
+//  2. router_select_kernel, one warp per token: sums the K parts, selects the
+//     top k + 1, weights, gap, the 32-token block's expert histogram and the
+//     shared-expert gate sigmoid(x . w_sg).  A call of at most kFuseTokens
+//     tokens also does the scatter's work here (offsets, permutation,
+//     generation re-check, GEMM groups), in the CTA that finishes last.
+#include "permute.cuh"
 
 namespace msi {
 
 namespace {
 
-constexpr int NTH = 256;  // 8 warps: all of them select top-k once the logits are in smem
-constexpr int RT_STAGES = 3;
-constexpr int RT_A = 128 * 64 * 2;                   // x tile (64 K)
-constexpr int RT_B = kRouterChunk * 64 * 2;          // one plane's chunk weight rows (64 K)
-constexpr int RT_STAGE = RT_A + 3 * RT_B;            // x tile + the three planes
-constexpr int RT_LLD = kRouterChunk + 1;             // padded logits row (floats)
-constexpr int RT_SMEM = 1024 + RT_STAGES * RT_STAGE + 256;
-static_assert(128 * RT_LLD * 4 <= RT_STAGES * RT_STAGE, "logits tile does not fit");
+constexpr int kCvtWarps = 16;                      // weight split, then the epilogue
+constexpr int kRlThreads = (kCvtWarps + 2) * 32;   // + TMA producer, MMA issuer
+constexpr int kXBytes = 128 * 64 * 2;              // x tile (64 of K)
 
-__device__ __forceinline__ void split3_body(const float* __restrict__ w, long long n,
-                                            __nv_bfloat16* __restrict__ out, int* status, Group* sh,
-                                            int* sh_total, int T, int shared_slot) {
-  // the forward's first kernel (status null: a prediction pass)
-  if (blockIdx.x == 0 && threadIdx.x == 0 && status != nullptr)
-    forward_begin(status, sh, sh_total, T, shared_slot);
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float v = w[i];
-    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-    const float r1 = v - __bfloat162float(hi);
-    const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-    const float r2 = r1 - __bfloat162float(mid);
-    out[i] = hi;
-    out[n + i] = mid;
-    out[2 * n + i] = __float2bfloat16_rn(r2);
-  }
+// STACK: the three planes are one MMA operand of 3 CH rows (two of 192 at
+// CH = 128) with an accumulator each, summed at the end: 4 or 8 MMAs per 64 of
+// K instead of 12.  A call's MMAs are then issue-bound no more (an MMA of 16
+// to 128 columns takes 85 to 107 cycles).
+template <int CH, bool STACK>
+struct RlCfg {
+  static constexpr int kPlane = CH * 128;          // one plane's rows (64 of K)
+  static constexpr int kStage = kXBytes + 3 * kPlane;
+  static constexpr int kStages = CH == 128 ? 3 : CH == 64 ? 5 : CH == 32 ? 7 : 8;
+  static constexpr int kSmem = 1024 + kStages * kStage + 256;
+  // the weight warps in groups that take the stages in turn, so that the
+  // loads' and the proxy fence's latencies overlap across the groups; a
+  // thread holds its group's next stage in registers.  No more groups than
+  // stages: a group that has filled stage `it` knows stages up to
+  // it - kStages to be consumed, and the next stage it tests must be at most
+  // one phase of its barrier beyond that (a parity cannot tell more).
+  static constexpr int kGroups = CH == 128 ? 2 : CH == 16 ? 8 : 4;
+  static constexpr int kGroupWarps = kCvtWarps / kGroups;
+  static constexpr int kVec = CH * 16 / (kGroupWarps * 32);  // 16-byte loads per thread and stage
+  static_assert(kGroups <= kStages && kVec * kGroupWarps * 32 == CH * 16, "weight groups");
+  static constexpr int kAcc = STACK ? 3 : 1;       // accumulators of CH columns
+  static constexpr int kCols = CH * kAcc <= 32 ? 32 : CH * kAcc <= 64 ? 64 : CH * kAcc <= 128 ? 128
+                               : CH * kAcc <= 256 ? 256 : 512;  // TMEM columns
+};
+
+// hi, mid and lo planes of two weights, as packed bf16 pairs
+__device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  hi = pack_bf16x2(a, b);
+  const float a1 = a - bf16_lo(hi), b1 = b - bf16_hi(hi);
+  mid = pack_bf16x2(a1, b1);
+  lo = pack_bf16x2(a1 - bf16_lo(mid), b1 - bf16_hi(mid));
 }
 
-__global__ void split3_kernel(const float* __restrict__ w, long long n, __nv_bfloat16* __restrict__ out,
-                              int* status, Group* sh, int* sh_total, int T, int shared_slot) {
-  split3_body(w, n, out, status, sh, sh_total, T, shared_slot);
-}
-
-// The same, plus the resident call's table copied to global memory: the
-// first warp of each block takes 32 entries, so the argument's entries are
-// read through many SMs' constant caches at once.
-__global__ void split3_table_kernel(const float* __restrict__ w, long long n,
-                                    __nv_bfloat16* __restrict__ out, int* status, Group* sh,
-                                    int* sh_total, int T, int shared_slot, const TableParams tp,
-                                    int* __restrict__ tab_slot,
-                                    unsigned long long* __restrict__ tab_expected) {
-  if (threadIdx.x < 32) {
-    for (int g = blockIdx.x * 32 + threadIdx.x; g < tp.E; g += gridDim.x * 32) {
-      tab_slot[g] = tp.slot[g];
-      tab_expected[g] = tp.expected[g];
-    }
-  }
-  split3_body(w, n, out, status, sh, sh_total, T, shared_slot);
-}
-
-// Selection order of the route event: logit descending, then expert id
-// ascending.  A logit maps to a 32-bit key with the same order (-0 counted as
-// +0), so a warp finds the best head of its lanes with one redux.sync max and
-// breaks a tie with one redux.sync min over the ids holding that key.
-__device__ __forceinline__ uint32_t logit_key(float v) {
-  uint32_t b = __float_as_uint(v);
-  if (b == 0x80000000u) b = 0u;
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float key_logit(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
-}
-
-// Sort one lane's N (key, id) pairs: key descending, id ascending.
-template <int N>
-__device__ __forceinline__ void sort_desc(uint32_t (&k)[N], int (&id)[N]) {
+// The weight warps' loop: the chunk's fp32 rows (src: its first row at the
+// CTA's first K; H apart), 64 of K per stage, into the three planes of the
+// stage.  ALIGNED: src is 16-byte aligned.
+template <int CH, bool STACK, bool ALIGNED>
+__device__ __forceinline__ void split_weights(const float* src, int H, int nstage, uint8_t* smem,
+                                              uint64_t* full, uint64_t* empty, volatile int* abort_flag,
+                                              long long lim) {
+  using C = RlCfg<CH, STACK>;
+  // thread: 16-byte piece of the rows row + 2 * kGroupWarps * i of the chunk
+  const int group = (threadIdx.x >> 5) / C::kGroupWarps;
+  const int gt = threadIdx.x - group * C::kGroupWarps * 32;
+  const int row = gt >> 4, piece = gt & 15;
+  constexpr int kRowStep = 2 * C::kGroupWarps;
+  src += (size_t)row * H + piece * 4;
+  float4 v[C::kVec];
+  auto load = [&](int it) {
 #pragma unroll
-  for (int i = 1; i < N; ++i) {
-#pragma unroll
-    for (int j = i; j > 0; --j) {
-      const bool sw = k[j] > k[j - 1] || (k[j] == k[j - 1] && id[j] < id[j - 1]);
-      const uint32_t tk = sw ? k[j - 1] : k[j];
-      const int ti = sw ? id[j - 1] : id[j];
-      k[j - 1] = sw ? k[j] : k[j - 1];
-      id[j - 1] = sw ? id[j] : id[j - 1];
-      k[j] = tk;
-      id[j] = ti;
+    for (int i = 0; i < C::kVec; ++i) {
+      const float* p = src + (size_t)(kRowStep * i) * H + it * 64;
+      v[i] = ALIGNED ? __ldg(reinterpret_cast<const float4*>(p))
+                     : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
     }
+  };
+  if (group < nstage) load(group);
+  for (int it = group; it < nstage; it += C::kGroups) {
+    const int s = it % C::kStages;
+    if (!mbar_wait(&empty[s], ((it / C::kStages) & 1) ^ 1, abort_flag, lim)) return;
+    const uint32_t st = smem_u32(smem + s * C::kStage) + kXBytes;
+#pragma unroll
+    for (int i = 0; i < C::kVec; ++i) {
+      uint2 pl[3];
+      split3(v[i].x, v[i].y, pl[0].x, pl[1].x, pl[2].x);
+      split3(v[i].z, v[i].w, pl[0].y, pl[1].y, pl[2].y);
+      const int r = row + kRowStep * i;
+      const uint32_t at = st + r * 128 + (((piece >> 1) ^ (r & 7)) << 4) + (piece & 1) * 8;
+#pragma unroll
+      for (int plane = 0; plane < 3; ++plane)
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + plane * C::kPlane), "r"(pl[plane].x),
+                     "r"(pl[plane].y)
+                     : "memory");
+    }
+    if (it + C::kGroups < nstage) load(it + C::kGroups);
+    fence_proxy_async_smem();  // before the tensor core's (async proxy) reads
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(&full[s]);
   }
 }
 
-// One selection round over the lanes' sorted heads: returns the winning key
-// and id (same in every lane); the lane that held it drops its head.
-template <int N>
-__device__ __forceinline__ void take_best(uint32_t (&k)[N], int (&id)[N], uint32_t& bk, int& bi) {
-  bk = __reduce_max_sync(0xffffffffu, k[0]);
-  bi = __reduce_min_sync(0xffffffffu, k[0] == bk ? id[0] : 0x7fffffff);
-  if (id[0] == bi && k[0] == bk) {
-#pragma unroll
-    for (int i = 0; i + 1 < N; ++i) {
-      k[i] = k[i + 1];
-      id[i] = id[i + 1];
-    }
-    k[N - 1] = 0u;  // below every logit's key
-    id[N - 1] = 0x7fffffff;
-  }
-}
-
-__global__ void __launch_bounds__(NTH, 1)
-    router_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
-                     const RouterTcArgs a) {
+template <int CH, bool STACK>
+__global__ void __launch_bounds__(kRlThreads, 1)
+    router_logits_kernel(const __grid_constant__ CUtensorMap tmX, const RouterTcArgs a,
+                         const __grid_constant__ TableParams tp) {
+  using C = RlCfg<CH, STACK>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + RT_STAGES * RT_STAGE);
-  uint64_t* empty = full + RT_STAGES;
-  uint64_t* tfull = empty + RT_STAGES;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStage);
+  uint64_t* empty = full + C::kStages;
+  uint64_t* tfull = empty + C::kStages;
   uint64_t* drain = tfull + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  uint64_t* never = drain + 1;  // no thread ever arrives here
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  int* ready_flag = const_cast<int*>(abort_flag) + 1;
-  uint64_t* never = reinterpret_cast<uint64_t*>(tmem_slot + 4);  // no thread ever arrives here
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int E = a.E;
-  const int ch = a.chunk;                 // experts per chunk
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // the chunks of one token tile are neighbours in launch order, so the x
   // tile is read from HBM once and from L2 by the other chunks
-  const int c = (int)(blockIdx.x % (unsigned)a.nchunk);  // chunk index
-  const int kblocks = a.H / 64;
-  const int nstage = kblocks;
-  const int m0 = (int)(blockIdx.x / (unsigned)a.nchunk) * 128;
+  int b = blockIdx.x;
+  const int c = b % a.nchunk;
+  b /= a.nchunk;
+  const int part = b % a.ksplit;
+  const int m0 = a.t0 + b / a.ksplit * 128;
+  const int nstage = a.H / 64 / a.ksplit;
+  const int kb0 = part * nstage;
   const long long lim = a.wait_limit;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < RT_STAGES; ++s) {
-      mbar_init(&full[s], 1);
+  if (tid == 0) {
+    for (int s = 0; s < C::kStages; ++s) {
+      mbar_init(&full[s], 1 + C::kGroupWarps);
       mbar_init(&empty[s], 1);
     }
     mbar_init(tfull, 1);
@@ -167,63 +160,77 @@ __global__ void __launch_bounds__(NTH, 1)
     mbar_init(never, 1);
     *abort_flag = 0;
     mbar_fence_init();
+    // the forward's first kernel begins it (status null: a prediction pass,
+    // or a later row chunk)
+    if (blockIdx.x == 0 && a.begin) {
+      forward_begin(a.status, a.sh, a.sh_total, a.T, tp.shared_slot);
+      *a.ticket = 0;
+    }
   }
-  if (warp == 4) {
-    tmem_alloc(tmem_slot, a.tmem_cols);
+  // the resident call's table, copied to global memory for the generation
+  // re-check: the entries are read through many SMs' constant caches at once
+  if (warp == kCvtWarps && a.begin)
+    for (int g = blockIdx.x * 32 + lane; g < tp.E; g += gridDim.x * 32) {
+      a.tab_slot[g] = tp.slot[g];
+      a.tab_expected[g] = tp.expected[g];
+    }
+  if (warp == kCvtWarps + 1) {
+    tmem_alloc(tmem_slot, C::kCols);
     tmem_relinquish();
-  }
-  if (warp == 5 && lane == 0) {
-    tma_prefetch(&tmX);
-    tma_prefetch(&tmW);
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 5) {
-    // ------------------------------------------------------------- TMA producer
+  if (warp == kCvtWarps) {
+    // ------------------------------------------------------------- x tiles (TMA)
     if (lane == 0) {
       int it = 0;
       for (; it < nstage; ++it) {
-        const int s = it % RT_STAGES;
-        const uint32_t ph = (it / RT_STAGES) & 1;
-        if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, lim)) break;
-        uint8_t* st = smem + s * RT_STAGE;
-        // x box: 128 rows of 64 bf16; weight boxes: `ch` rows of 64 bf16 per plane
-        mbar_arrive_expect_tx(&full[s], RT_A + 3 * ch * 128);
-        tma_load_2d(st, &tmX, &full[s], it * 64, m0);
-#pragma unroll
-        for (int plane = 0; plane < 3; ++plane)
-          tma_load_2d(st + RT_A + plane * RT_B, &tmW, &full[s], it * 64, plane * E + c * ch);
+        const int s = it % C::kStages;
+        if (!mbar_wait(&empty[s], ((it / C::kStages) & 1) ^ 1, abort_flag, lim)) break;
+        mbar_arrive_expect_tx(&full[s], kXBytes);
+        tma_load_2d(smem + s * C::kStage, &tmX, &full[s], (kb0 + it) * 64, m0);
       }
+      // on abort the armed loads land before shared memory is released (a
+      // stage's barrier may still lack the weight arrivals: bounded)
       if (*abort_flag) {
-        for (int d = 0; d < RT_STAGES && it - 1 - d >= 0; ++d) {
+        for (int d = 0; d < C::kStages && it - 1 - d >= 0; ++d) {
           const int j = it - 1 - d;
           const long long t0 = clock64();
-          while (!mbar_try_wait(&full[j % RT_STAGES], (j / RT_STAGES) & 1) && clock64() - t0 < kDrainCycles) {
+          while (!mbar_try_wait(&full[j % C::kStages], (j / C::kStages) & 1) && clock64() - t0 < kDrainCycles) {
           }
         }
       }
     }
-  } else if (warp == 4) {
+  } else if (warp == kCvtWarps + 1) {
     // ------------------------------------------------------------- MMA issuer
     if (lane == 0) {
       bool ok = true;
-      const uint32_t idesc = idesc_bf16(128, ch);
       for (int it = 0; it < nstage; ++it) {
-        const int s = it % RT_STAGES;
-        const uint32_t ph = (it / RT_STAGES) & 1;
-        if (!mbar_wait(&full[s], ph, abort_flag, lim)) { ok = false; break; }
+        const int s = it % C::kStages;
+        if (!mbar_wait(&full[s], (it / C::kStages) & 1, abort_flag, lim)) { ok = false; break; }
         tc_fence_after();
-        const uint8_t* st = smem + s * RT_STAGE;
-        const uint64_t ad = sw128_desc(smem_u32(st));
+        const uint32_t st = smem_u32(smem + s * C::kStage);
+        const uint64_t ad = sw128_desc(st);
+        if (STACK) {
+          constexpr int kN = CH == 128 ? 192 : 3 * CH;  // rows per MMA
 #pragma unroll
-        for (int plane = 0; plane < 3; ++plane) {
-          const uint64_t bd = sw128_desc(smem_u32(st + RT_A + plane * RT_B));
+          for (int kk = 0; kk < 4; ++kk) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            umma_bf16(tmem_base, ad + 2 * kk, bd + 2 * kk, idesc, (it | plane | kk) != 0);
+            for (int n0 = 0; n0 < 3 * CH; n0 += kN)
+              umma_bf16(tmem_base + n0, ad + 2 * kk, sw128_desc(st + kXBytes + n0 * 128) + 2 * kk,
+                        idesc_bf16(128, kN), (it | kk) != 0);
+          }
+        } else {
+#pragma unroll
+          for (int plane = 0; plane < 3; ++plane) {
+            const uint64_t bd = sw128_desc(st + kXBytes + plane * C::kPlane);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              umma_bf16(tmem_base, ad + 2 * kk, bd + 2 * kk, idesc_bf16(128, CH), (it | plane | kk) != 0);
+          }
         }
         umma_commit(&empty[s]);
       }
@@ -233,74 +240,42 @@ __global__ void __launch_bounds__(NTH, 1)
       while (!mbar_try_wait(drain, 0) && clock64() - t0 < kDrainCycles) {
       }
     }
-  } else if (warp < 4) {
-    // ------------------------------------------------------------- epilogue
-    // Chunk logits TMEM -> shared memory (the stage buffers are free once the
-    // MMA loop is done; rows padded so the 32 lanes' column writes fall into
-    // distinct banks).
-    if (a.stall && threadIdx.x == 0) mbar_wait(never, 0, abort_flag, lim);  // runs out: abort
+  } else {
+    // ------------------------------------------------------------- weights
+    const float* src = a.wr + (size_t)c * CH * a.H + (size_t)kb0 * 64;
+    if ((reinterpret_cast<uintptr_t>(a.wr) & 15) == 0)
+      split_weights<CH, STACK, true>(src, a.H, nstage, smem, full, empty, abort_flag, lim);
+    else
+      split_weights<CH, STACK, false>(src, a.H, nstage, smem, full, empty, abort_flag, lim);
+    // ------------------------------------------------------------- logits out
+    if (a.stall && tid == 0) mbar_wait(never, 0, abort_flag, lim);  // runs out: abort
     const bool ready = __all_sync(0xffffffffu, mbar_wait(tfull, 0, abort_flag, lim)) && !*abort_flag;
     tc_fence_after();
-    float* L = reinterpret_cast<float*>(smem);
-    if (ready) {
-      const uint32_t tb = tmem_base + ((uint32_t)(warp * 32) << 16);
-      float* row = L + (size_t)(warp * 32 + lane) * RT_LLD;
-      for (int e0 = 0; e0 < ch; e0 += 16) {
-        uint32_t v[16];
-        tmem_ld16(tb + e0, v);
-        tmem_ld_wait(v);
+    const int t = m0 + (warp & 3) * 32 + lane;  // TMEM lane: the token
+    // the four warps of a lane quarter share the columns, 16 at least each
+    constexpr int kPer = CH >= 64 ? CH / 4 : 16;
+    const int c0 = (warp >> 2) * kPer;
+    if (ready && c0 < CH) {
+      const uint32_t tb = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + c0;
+      float* dst = a.logits + ((size_t)part * a.rows + (t - a.t0)) * a.E + c * CH + c0;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) row[e0 + j] = __uint_as_float(v[j]);
-      }
-    }
-    if (threadIdx.x == 0) *ready_flag = ready ? 1 : 0;
-  }
-
-  tc_fence_before();
-  __syncthreads();
-  if (*ready_flag) {
-    // ------------------------------------------------------------- top-k
-    // every warp: its 16 tokens' top k+1 in the chunk, four tokens at a time
-    const float* L = reinterpret_cast<const float*>(smem);
-    const int kp = a.kp;  // candidates per chunk: min(k + 1, chunk)
-    constexpr int NL = kRouterChunk / 32;  // logits per lane and token
-    for (int q0 = warp * 16; q0 < warp * 16 + 16; q0 += 4) {
-      uint32_t kk[4][NL];
-      int id[4][NL];
-      float my_v[4];
-      int my_i[4];
+      for (int e0 = 0; e0 < kPer; e0 += 16) {
+        uint32_t r[16];
+        tmem_ld16(tb + e0, r);
+        tmem_ld_wait(r);
+        if (STACK) {
+          uint32_t mid[16], lo[16];
+          tmem_ld16(tb + CH + e0, mid);
+          tmem_ld16(tb + 2 * CH + e0, lo);
+          tmem_ld_wait(mid);
+          tmem_ld_wait(lo);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float* row = L + (size_t)(q0 + u) * RT_LLD;
-#pragma unroll
-        for (int i = 0; i < NL; ++i) {
-          const int e = lane + 32 * i;
-          kk[u][i] = e < ch ? logit_key(row[e]) : 0u;
-          id[u][i] = e < ch ? e : 0x7fffffff;
+          for (int i = 0; i < 16; ++i)
+            r[i] = __float_as_uint(__uint_as_float(r[i]) + (__uint_as_float(mid[i]) + __uint_as_float(lo[i])));
         }
-        sort_desc(kk[u], id[u]);
-        my_v[u] = -INFINITY;
-        my_i[u] = 0x7fffffff;
-      }
-      for (int rr = 0; rr < kp; ++rr) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          uint32_t bk;
-          int bi;
-          take_best(kk[u], id[u], bk, bi);
-          if (rr == lane) {
-            my_v[u] = key_logit(bk);
-            my_i[u] = c * ch + bi;  // global expert id
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = m0 + q0 + u;
-        if (lane < kp && t < a.T) {
-          const size_t o = ((size_t)t * a.nchunk + c) * kp + lane;
-          a.cand_v[o] = my_v[u];
-          a.cand_i[o] = my_i[u];
+        if (t < a.T && t < a.t0 + a.rows) {
+          st_global_v8(dst + e0, r);
+          st_global_v8(dst + e0 + 8, r + 8);
         }
       }
     }
@@ -308,160 +283,347 @@ __global__ void __launch_bounds__(NTH, 1)
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 4) {
+  if (warp == kCvtWarps + 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, a.tmem_cols);
+    tmem_dealloc(tmem_base, C::kCols);
   }
-  if (threadIdx.x == 0 && *abort_flag) atomicCAS(a.status, 0, (int)MSI_ERR_TIMEOUT);
+  if (tid == 0 && *abort_flag) atomicCAS(a.status, 0, (int)MSI_ERR_TIMEOUT);
 }
 
-// One CTA per 32-token block (sixteen warps, two tokens each, selected
-// together): top-(k+1) of the union of the chunks' candidates, the route
-// event (ids, weights, gap), the block's expert histogram (one row of bcount
-// for the permutation) and, when the layer has a shared expert, its gate
-// sigmoid(x . w_sg).
-constexpr int kMergeTPW = 2;                     // tokens per warp
-constexpr int kMergeThreads = 32 / kMergeTPW * 32;  // one CTA per 32-token block
+// Selection order of the route event: logit descending, then expert id
+// ascending.  A logit maps to a 32-bit key with the same order (-0 counted as
+// +0; never 0, which stands for no entry); the key above the complement of the
+// id is a 64-bit word that is larger the earlier its entry is selected, and no
+// two entries share one.
+__device__ __forceinline__ uint32_t logit_key(float v) {
+  const int b = __float_as_int(v + 0.0f);
+  return max((uint32_t)(b ^ ((b >> 31) | (int)0x80000000)), 1u);
+}
+__device__ __forceinline__ float key_logit(uint32_t k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
+}
+__device__ __forceinline__ unsigned long long entry_word(uint32_t key, int id) {
+  return ((unsigned long long)key << 32) | (uint32_t)~id;
+}
 
-__global__ void __launch_bounds__(kMergeThreads) router_merge_kernel(const RouterTcArgs a) {
-  constexpr int U = kMergeTPW;
-  __shared__ int hist[kMaxExperts];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+constexpr int kCand = 64;  // candidates ranked together
+struct SelectScratch {     // shared memory of one warp
+  uint4 head[8];
+  unsigned long long word[kCand];
+  unsigned long long best[32];
+  int id[kCand];
+};
+
+// One warp, one token: ids, weights and gap of token t; returns lane j's
+// selected id (j < k).  Lane l holds the experts 128 i + 4 l + c (c < 4,
+// i < NV).  The (k + 1)-th largest of the 32 lanes' best logits bounds the
+// (k + 1)-th largest of all from below, so the selection is among the entries
+// not below it: usually a few more than k + 1.  Each of those finds its rank
+// by counting the larger ones.  Every step is a handful of independent
+// compares, where k + 1 rounds of a warp argmax are one dependent chain; the
+// kernel is bound by its instructions, and by their latency for few tokens.
+template <int NV>
+__device__ __forceinline__ int select_token(const RouterTcArgs& a, int t, int lane, SelectScratch& sc) {
   const int E = a.E, k = a.k;
-  const int ncand = a.nchunk * a.kp;  // <= 160
-  for (int e = threadIdx.x; e < E; e += blockDim.x) hist[e] = 0;
-  __syncthreads();
-  const int tw = blockIdx.x * 32 + warp * U;  // this warp's first token
-  {
-    uint32_t kk[U][5];
-    int id[U][5];
+  const size_t part_stride = (size_t)a.rows * E;
+  const float* L = a.logits + (size_t)(t - a.t0) * E;
+  float4 v[NV];
+  auto load = [&](const float* P, float4 (&d)[NV]) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int t = tw + u;
-#pragma unroll
-      for (int i = 0; i < 5; ++i) {
-        const int j = lane + 32 * i;
-        const bool in = t < a.T && j < ncand;
-        const int cid = in ? a.cand_i[(size_t)t * ncand + j] : -1;
-        const bool real = cid >= 0 && cid < E;  // an aborted router leaves no valid candidate
-        kk[u][i] = real ? logit_key(a.cand_v[(size_t)t * ncand + j]) : 0u;
-        id[u][i] = real ? cid : 0x7fffffff;
-      }
-      sort_desc(kk[u], id[u]);
-    }
-    float my_v[U], next_v[U];
-    int my_i[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      my_v[u] = -INFINITY;
-      next_v[u] = -INFINITY;
-      my_i[u] = 0;
-    }
-    const int rounds = min(k + 1, E);
-    for (int rr = 0; rr < rounds; ++rr) {
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        uint32_t bk;
-        int bi;
-        take_best(kk[u], id[u], bk, bi);
-        const float bv = bk == 0u ? -INFINITY : key_logit(bk);
-        if (rr == lane) {
-          my_v[u] = bv;
-          my_i[u] = bi;
-        }
-        if (rr == k) next_v[u] = bv;
-      }
+    for (int i = 0; i < NV; ++i)
+      d[i] = 128 * i + 4 * lane < E ? *reinterpret_cast<const float4*>(P + 128 * i + 4 * lane)
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  // the K parts in a fixed order: p0 + p1 + (p2 + p3)
+  load(L, v);
+  if (a.ksplit >= 2) {
+    float4 p1[NV], p2[NV], p3[NV];
+    load(L + part_stride, p1);
+    if (a.ksplit == 4) {
+      load(L + 2 * part_stride, p2);
+      load(L + 3 * part_stride, p3);
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int t = tw + u;
-      const float l0 = __shfl_sync(0xffffffffu, my_v[u], 0);
-      const float ex = (lane < k) ? expf(my_v[u] - l0) : 0.f;
-      float sum = ex;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-      const float lk1 = __shfl_sync(0xffffffffu, my_v[u], k - 1);
-      if (t < a.T) {
-        if (lane < k) {
-          // an aborted router leaves no valid candidate: expert 0 stands in,
-          // counted like any id, so that the permutation stays a bijection
-          // (the status word already fails the call)
-          const bool real = my_i[u] >= 0 && my_i[u] < E;
-          const int id = real ? my_i[u] : 0;
-          a.ids[(size_t)t * k + lane] = id;
-          a.weights[(size_t)t * k + lane] = ex / sum;
-          atomicAdd(&hist[id], 1);
-        }
-        if (a.gap != nullptr && lane == 0) a.gap[t] = (k < E) ? (lk1 - next_v[u]) : INFINITY;
+    for (int i = 0; i < NV; ++i) {
+      v[i].x += p1[i].x; v[i].y += p1[i].y; v[i].z += p1[i].z; v[i].w += p1[i].w;
+      if (a.ksplit == 4) {
+        v[i].x += p2[i].x + p3[i].x; v[i].y += p2[i].y + p3[i].y;
+        v[i].z += p2[i].z + p3[i].z; v[i].w += p2[i].w + p3[i].w;
       }
     }
   }
-  if (a.wsg != nullptr) {
-    // shared-expert gate of the warp's tokens, dot products interleaved
-    float sum[U];
+  uint32_t key[4 * NV], hk = 0u;
 #pragma unroll
-    for (int u = 0; u < U; ++u) sum[u] = 0.f;
+  for (int i = 0; i < NV; ++i) {
+    const bool in = 128 * i + 4 * lane < E;
+    const float w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      key[4 * i + c] = in ? logit_key(w[c]) : 0u;
+      hk = max(hk, key[4 * i + c]);
+    }
+  }
+  const int rounds = min(k + 1, E);
+  __syncwarp();  // the previous token's readers are done
+  reinterpret_cast<uint32_t*>(sc.head)[lane] = hk;
+  __syncwarp();
+  int above = 0;  // lanes whose best is larger
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint4 q = sc.head[j];
+    above += (q.x > hk) + (q.y > hk) + (q.z > hk) + (q.w > hk);
+  }
+  // at least min(rounds, 32) lanes hold an entry not below the bound, or all
+  // lanes with entries do
+  const uint32_t bound = max(__reduce_min_sync(0xffffffffu, above < rounds ? hk : 0xFFFFFFFFu), 1u);
+  uint32_t mask = 0u;
+#pragma unroll
+  for (int j = 0; j < 4 * NV; ++j) mask |= key[j] >= bound ? 1u << j : 0u;
+  int at = __popc(mask);
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, at, off);
+    if (lane >= off) at += o;
+  }
+  const int n = __shfl_sync(0xffffffffu, at, 31);
+  at -= __popc(mask);
+  if (n <= kCand) {
+    for (; mask != 0u; mask &= mask - 1u) {
+      const int j = __ffs(mask) - 1;
+      sc.id[at++] = 128 * (j >> 2) + 4 * lane + (j & 3);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int u = 0; u < n; u += 32) {
+      const int q = u + lane;
+      if (q < n) {
+        const int e = sc.id[q];
+        float x = L[e];
+        if (a.ksplit >= 2) x += L[part_stride + e];
+        if (a.ksplit == 4) x += L[2 * part_stride + e] + L[3 * part_stride + e];
+        sc.word[q] = entry_word(logit_key(x), e);
+      }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int u = 0; u < n; u += 32) {
+      const unsigned long long c = u + lane < n ? sc.word[u + lane] : 0ull;
+      int r = 0;
 #pragma unroll 4
-    for (int h = lane * 8; h < a.H; h += 256) {
-      const float4 w0 = __ldg(reinterpret_cast<const float4*>(a.wsg + h));
-      const float4 w1 = __ldg(reinterpret_cast<const float4*>(a.wsg + h + 4));
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (tw + u >= a.T) continue;
-        const uint4 xv = __ldg(reinterpret_cast<const uint4*>(a.x + (size_t)(tw + u) * a.H + h));
-        float s = sum[u];
-        s = fmaf(bf16_lo(xv.x), w0.x, s);
-        s = fmaf(bf16_hi(xv.x), w0.y, s);
-        s = fmaf(bf16_lo(xv.y), w0.z, s);
-        s = fmaf(bf16_hi(xv.y), w0.w, s);
-        s = fmaf(bf16_lo(xv.z), w1.x, s);
-        s = fmaf(bf16_hi(xv.z), w1.y, s);
-        s = fmaf(bf16_lo(xv.w), w1.z, s);
-        s = fmaf(bf16_hi(xv.w), w1.w, s);
-        sum[u] = s;
-      }
+      for (int j = 0; j < n; ++j) r += sc.word[j] > c;
+      if (u + lane < n && r < rounds) sc.best[r] = c;
     }
+  } else {
+    // many entries share few lanes, or one logit: a warp argmax per round
+    unsigned long long last = ~0ull;
+#pragma unroll 1
+    for (int r = 0; r < rounds; ++r) {
+      unsigned long long b = 0ull;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      float s = sum[u];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      if (lane == 0 && tw + u < a.T) a.sg[tw + u] = 1.0f / (1.0f + expf(-s));
+      for (int j = 0; j < 4 * NV; ++j) {
+        const unsigned long long w = entry_word(key[j], 128 * (j >> 2) + 4 * lane + (j & 3));
+        if (key[j] != 0u && w < last && w > b) b = w;
+      }
+#pragma unroll 1
+      for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, b, off);
+        b = o > b ? o : b;
+      }
+      if (lane == 0) sc.best[r] = b;
+      last = b;
     }
   }
+  __syncwarp();
+  const unsigned long long mine = sc.best[min(lane, rounds - 1)];
+  const int my_i = (int)~(uint32_t)mine;
+  const float my_v = key_logit((uint32_t)(mine >> 32));
+  const float l0 = __shfl_sync(0xffffffffu, my_v, 0);
+  const float ex = lane < k ? expf(my_v - l0) : 0.f;
+  float sum = ex;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  const float lk = __shfl_sync(0xffffffffu, my_v, k - 1);
+  const float lk1 = __shfl_sync(0xffffffffu, my_v, k);
+  if (lane < k) {
+    a.ids[(size_t)t * k + lane] = my_i;
+    a.weights[(size_t)t * k + lane] = ex / sum;
+  }
+  if (a.gap != nullptr && lane == 0) a.gap[t] = (k < E) ? (lk - lk1) : INFINITY;
+  return my_i;
+}
+
+// sigmoid(x[t] . w_sg) by one warp
+__device__ __forceinline__ void shared_gate(const RouterTcArgs& a, int t, int lane) {
+  float s = 0.f;
+#pragma unroll 4
+  for (int h = lane * 8; h < a.H; h += 256) {
+    const float4 w0 = __ldg(reinterpret_cast<const float4*>(a.wsg + h));
+    const float4 w1 = __ldg(reinterpret_cast<const float4*>(a.wsg + h + 4));
+    const uint4 xv = __ldg(reinterpret_cast<const uint4*>(a.x + (size_t)t * a.H + h));
+    s = fmaf(bf16_lo(xv.x), w0.x, s);
+    s = fmaf(bf16_hi(xv.x), w0.y, s);
+    s = fmaf(bf16_lo(xv.y), w0.z, s);
+    s = fmaf(bf16_hi(xv.y), w0.w, s);
+    s = fmaf(bf16_lo(xv.z), w1.x, s);
+    s = fmaf(bf16_hi(xv.z), w1.y, s);
+    s = fmaf(bf16_lo(xv.w), w1.z, s);
+    s = fmaf(bf16_hi(xv.w), w1.w, s);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if (lane == 0) a.sg[t] = 1.0f / (1.0f + expf(-s));
+}
+
+// One CTA per 32-token block, two tokens a warp; the block's histogram is one
+// row of bcount for the permutation.
+template <int NV>
+__global__ void __launch_bounds__(512, 2) router_select_kernel(const RouterTcArgs a) {
+  __shared__ int hist[kMaxExperts];
+  __shared__ SelectScratch scratch[16];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int e = threadIdx.x; e < a.E; e += blockDim.x) hist[e] = 0;
   __syncthreads();
-  for (int e = threadIdx.x; e < E; e += blockDim.x) a.bcount[(size_t)blockIdx.x * E + e] = hist[e];
+#pragma unroll 1
+  for (int u = 0; u < 2; ++u) {
+    const int t = a.t0 + blockIdx.x * 32 + u * 16 + warp;
+    if (t >= a.T) break;
+    const int id = select_token<NV>(a, t, lane, scratch[warp]);
+    if (lane < a.k) atomicAdd(&hist[id], 1);
+    if (a.wsg != nullptr) shared_gate(a, t, lane);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < a.E; e += blockDim.x)
+    a.bcount[(size_t)(a.t0 / 32 + blockIdx.x) * a.E + e] = hist[e];
+}
+
+// A call of at most kFuseTokens tokens: eight tokens a CTA (selection on eight
+// warps, the gates on the other eight), and the CTA that finishes last does
+// the scatter's work for the whole call: histogram, permutation, generation
+// re-check and GEMM groups.  A token names an expert at most once, so an
+// expert's rows are the set bits of its token mask: counts and stable ranks
+// are population counts.  Latency is all there is to it: one launch instead
+// of two or three, and the slots' words are loaded before the ids are known.
+template <int NV>
+__global__ void __launch_bounds__(512, 2) router_select_scatter_kernel(const RouterTcArgs a,
+                                                                       const ScatterArgs s) {
+  constexpr int kTok = 8;
+  __shared__ unsigned mask[kFuseTokens / 32][kMaxExperts];
+  __shared__ int offs[kMaxExperts];
+  __shared__ int tmp[32];
+  __shared__ int s_last;
+  __shared__ SelectScratch scratch[kTok];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int e = tid;
+  int slot = -1, code = 0;
+  if (s.tab_slot != nullptr && e < a.E) {
+    slot = s.tab_slot[e];
+    code = check_code(s.genwords, slot, s.layer, e, s.tab_expected[e]);
+  }
+  const int t = blockIdx.x * kTok + (warp & (kTok - 1));
+  if (t < a.T) {
+    if (warp < kTok) select_token<NV>(a, t, lane, scratch[warp]);
+    else if (a.wsg != nullptr) shared_gate(a, t, lane);
+  }
+  __threadfence();  // the ids, before the ticket
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(s.ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const int nw = (a.T + 31) / 32;
+  for (int w = 0; w < nw; ++w) mask[w][tid] = 0u;
+  for (int r = tid; r < s.n_ready; r += blockDim.x) s.ready[r] = 0;
+  __syncthreads();
+  const int n = a.T * a.k;
+  for (int f = tid; f < n; f += blockDim.x) {
+    const int tok = f / a.k;
+    atomicOr(&mask[tok >> 5][__ldcg(&a.ids[f])], 1u << (tok & 31));
+  }
+  __syncthreads();
+  int cnt = 0;
+  if (e < a.E)
+    for (int w = 0; w < nw; ++w) cnt += __popc(mask[w][e]);
+  int total;
+  const int base = block_excl_scan(cnt, tmp, &total);
+  offs[e] = base;
+  if (e < a.E) {
+    s.offsets[e] = base;
+    s.counts_out[e] = cnt;
+  }
+  if (tid == 0) s.offsets[a.E] = total;
+  __syncthreads();
+  for (int f = tid; f < n; f += blockDim.x) {
+    const int tok = f / a.k, id = __ldcg(&a.ids[f]), w = tok >> 5;
+    int pos = offs[id] + __popc(mask[w][id] & ((1u << (tok & 31)) - 1u));  // + the expert's earlier tokens
+    for (int q = 0; q < w; ++q) pos += __popc(mask[q][id]);
+    s.perm[pos] = f;
+    s.inv[f] = pos;
+  }
+  if (s.tab_slot != nullptr) build_groups(s, e, cnt, base, slot, cnt > 0 ? code : 0, tmp);
+}
+
+template <int CH, bool STACK>
+cudaError_t launch_logits(const CUtensorMap& tmX, const RouterTcArgs& a, const TableParams& tp, cudaStream_t s) {
+  static std::atomic<unsigned long long> attr_done{0};
+  constexpr int smem = RlCfg<CH, STACK>::kSmem;
+  cudaError_t e = smem_attr_once(router_logits_kernel<CH, STACK>, smem, attr_done);
+  if (e != cudaSuccess) return e;
+  const unsigned grid = (unsigned)((a.rows + 127) / 128) * a.nchunk * a.ksplit;
+  router_logits_kernel<CH, STACK><<<grid, kRlThreads, smem, s>>>(tmX, a, tp);
+  return cudaGetLastError();
+}
+
+template <int NV>
+void select_nv(const RouterTcArgs& a, const ScatterArgs* sa, cudaStream_t s) {
+  if (sa != nullptr) router_select_scatter_kernel<NV><<<(a.T + 7) / 8, 512, 0, s>>>(a, *sa);
+  else router_select_kernel<NV><<<(a.rows + 31) / 32, 512, 0, s>>>(a);
 }
 
 }  // namespace
 
-cudaError_t launch_split3(const float* w, long long n, __nv_bfloat16* out, int* status, Group* sh,
-                          int* sh_total, int T, int shared_slot, const TableParams* tp,
-                          int* tab_slot, unsigned long long* tab_expected, cudaStream_t s) {
-  const long long want = (n + 255) / 256;
-  const int grid = (int)(want < 152 * 8 ? want : 152 * 8);
-  if (tp != nullptr)
-    split3_table_kernel<<<grid, 256, 0, s>>>(w, n, out, status, sh, sh_total, T, shared_slot, *tp,
-                                             tab_slot, tab_expected);
-  else
-    split3_kernel<<<grid, 256, 0, s>>>(w, n, out, status, sh, sh_total, T, shared_slot);
-  return cudaGetLastError();
+// Expert chunk and K split of a call of T rows: the cut with the least time by
+// a fit of the measured launches (event-timed over 1 to 8,192 rows, 512
+// experts, H 2,048, every chunk and split): about 6 us a CTA, then 0.25 us +
+// 2 ns per expert of its chunk for each 64 of K, per round of CTAs on the SMs;
+// every K part adds reads to the selection.  One token: 16 experts x 4 parts
+// 7.0 us (128 experts, one part: 24); 600 tokens: 128 x 4, 11.4 us (16 x 1, two
+// rounds: 30); 4,096 tokens: 128 x 1, 27.5 us.
+// Planes stacked up to kStackTokens: 28 against 30 us at 4,096 tokens, 1 to 9
+// us less at smaller chunks.
+RouterSplit router_split(int T, int E, int sms) {
+  const int mt = (T + 127) / 128;
+  RouterSplit best{16, 1, false};
+  double cost = 1e30;
+  for (int ch = 16; ch <= 128 && E % ch == 0; ch *= 2)
+    for (int ks = 1; ks <= 4; ks *= 2) {
+      const int waves = (int)(((long long)mt * (E / ch) * ks + sms - 1) / sms);
+      const double c = waves * (6.0 + 32.0 / ks * (0.25 + ch * 0.002)) + 0.5 * ks;
+      if (c < cost) {
+        cost = c;
+        best.chunk = ch;
+        best.ksplit = ks;
+      }
+    }
+  best.stack = T <= kStackTokens;
+  return best;
 }
 
-cudaError_t launch_router_tc(const CUtensorMap& tmX, const CUtensorMap& tmW, const RouterTcArgs& a,
-                             cudaStream_t s) {
-  static std::atomic<unsigned long long> attr_done{0};
-  {
-    cudaError_t e = smem_attr_once(router_tc_kernel, RT_SMEM, attr_done);
-    if (e != cudaSuccess) return e;
+cudaError_t launch_router_logits(const CUtensorMap& tmX, const RouterTcArgs& a, const TableParams& tp,
+                                 cudaStream_t s) {
+  switch (a.chunk) {
+    case 16: return a.stack ? launch_logits<16, true>(tmX, a, tp, s) : launch_logits<16, false>(tmX, a, tp, s);
+    case 32: return a.stack ? launch_logits<32, true>(tmX, a, tp, s) : launch_logits<32, false>(tmX, a, tp, s);
+    case 64: return a.stack ? launch_logits<64, true>(tmX, a, tp, s) : launch_logits<64, false>(tmX, a, tp, s);
+    default: return a.stack ? launch_logits<128, true>(tmX, a, tp, s) : launch_logits<128, false>(tmX, a, tp, s);
   }
-  const int nb = (a.T + 127) / 128;
-  if (nb == 0) return cudaSuccess;
-  router_tc_kernel<<<(unsigned)nb * (unsigned)a.nchunk, NTH, RT_SMEM, s>>>(tmX, tmW, a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  router_merge_kernel<<<(a.T + 31) / 32, kMergeThreads, 0, s>>>(a);
+}
+
+cudaError_t launch_router_select(const RouterTcArgs& a, const ScatterArgs* sa, cudaStream_t s) {
+  const int nv = (a.E + 127) / 128;
+  if (nv <= 1) select_nv<1>(a, sa, s);
+  else if (nv <= 2) select_nv<2>(a, sa, s);
+  else select_nv<4>(a, sa, s);
   return cudaGetLastError();
 }
 
