@@ -425,6 +425,28 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
       : "memory");
 }
 
+// One lane of a converged warp, the same one each time.  The MMA warps run
+// their loops with all lanes and issue under this predicate: in a branch on
+// the lane id the operands of every MMA are moved register by register into
+// uniform ones, which held a K step's four MMAs to 600 to 900 cycles where the
+// tensor core takes 200 to 512.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+// A value that every lane holds, as one the compiler can see to be uniform.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_max_sync(0xffffffffu, v); }
+// A wait of the whole warp, with one answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                               long long limit) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit));
+}
+
 // D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                           uint32_t idesc, uint32_t accumulate) {

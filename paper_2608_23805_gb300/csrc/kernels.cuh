@@ -67,7 +67,7 @@ struct RouterSplit {
   int chunk, ksplit;
   bool stack;
 };
-constexpr int kStackTokens = 4096;  // longest call with the planes stacked (router_tc.cu)
+constexpr int kSplitTokens = 64;  // longest call with K parts and stacked planes (router_tc.cu)
 RouterSplit router_split(int T, int E, int sms);
 
 struct ScanArgs {

@@ -43,8 +43,7 @@ constexpr int kXBytes = 128 * 64 * 2;              // x tile (64 of K)
 
 // STACK: the three planes are one MMA operand of 3 CH rows (two of 192 at
 // CH = 128) with an accumulator each, summed at the end: 4 or 8 MMAs per 64 of
-// K instead of 12.  A call's MMAs are then issue-bound no more (an MMA of 16
-// to 128 columns takes 85 to 107 cycles).
+// K instead of 12 (an MMA of up to 96 columns takes 48 cycles, of 128 64).
 template <int CH, bool STACK>
 struct RlCfg {
   static constexpr int kPlane = CH * 128;          // one plane's rows (64 of K)
@@ -206,22 +205,25 @@ __global__ void __launch_bounds__(kRlThreads, 1)
     }
   } else if (warp == kCvtWarps + 1) {
     // ------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      bool ok = true;
-      for (int it = 0; it < nstage; ++it) {
-        const int s = it % C::kStages;
-        if (!mbar_wait(&full[s], (it / C::kStages) & 1, abort_flag, lim)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t st = smem_u32(smem + s * C::kStage);
-        const uint64_t ad = sw128_desc(st);
+    // (all lanes wait, one elected lane issues)
+    bool ok = true;
+    const uint32_t tm = uniform(tmem_base);
+    uint32_t s = 0, ph = 0;
+    for (int it = 0; it < nstage; ++it) {
+      ok = mbar_wait_warp(&full[s], ph, abort_flag, lim);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t st = smem_u32(smem + s * C::kStage);
+      const uint64_t ad = sw128_desc(st);
+      if (elect_one()) {
         if (STACK) {
           constexpr int kN = CH == 128 ? 192 : 3 * CH;  // rows per MMA
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
 #pragma unroll
             for (int n0 = 0; n0 < 3 * CH; n0 += kN)
-              umma_bf16(tmem_base + n0, ad + 2 * kk, sw128_desc(st + kXBytes + n0 * 128) + 2 * kk,
-                        idesc_bf16(128, kN), (it | kk) != 0);
+              umma_bf16(tm + n0, ad + 2 * kk, sw128_desc(st + kXBytes + n0 * 128) + 2 * kk, idesc_bf16(128, kN),
+                        (it | kk) != 0);
           }
         } else {
 #pragma unroll
@@ -229,11 +231,19 @@ __global__ void __launch_bounds__(kRlThreads, 1)
             const uint64_t bd = sw128_desc(st + kXBytes + plane * C::kPlane);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              umma_bf16(tmem_base, ad + 2 * kk, bd + 2 * kk, idesc_bf16(128, CH), (it | plane | kk) != 0);
+              umma_bf16(tm, ad + 2 * kk, bd + 2 * kk, idesc_bf16(128, CH), (it | plane | kk) != 0);
           }
         }
         umma_commit(&empty[s]);
       }
+      __syncwarp();
+      if (++s == C::kStages) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
+    __syncwarp();
+    if (elect_one()) {
       if (ok) umma_commit(tfull);
       umma_commit(drain);
       const long long t0 = clock64();
@@ -585,18 +595,19 @@ void select_nv(const RouterTcArgs& a, const ScatterArgs* sa, cudaStream_t s) {
 // Expert chunk and K split of a call of T rows: the cut with the least time by
 // a fit of the measured launches (event-timed over 1 to 8,192 rows, 512
 // experts, H 2,048, every chunk and split): about 6 us a CTA, then 0.25 us +
-// 2 ns per expert of its chunk for each 64 of K, per round of CTAs on the SMs;
-// every K part adds reads to the selection.  One token: 16 experts x 4 parts
-// 7.0 us (128 experts, one part: 24); 600 tokens: 128 x 4, 11.4 us (16 x 1, two
-// rounds: 30); 4,096 tokens: 128 x 1, 27.5 us.
-// Planes stacked up to kStackTokens: 28 against 30 us at 4,096 tokens, 1 to 9
-// us less at smaller chunks.
+// 2 ns per expert of its chunk for each 64 of K, per round of CTAs on the SMs.
+// One token: 16 experts x 4 parts 7.0 us (128 experts, one part: 24).
+// K parts and stacked planes sum a logit in another order than one chain over
+// K.  That moves it by about 1e-6, enough to swap a pair of experts that close
+// on one row in some ten thousand, so it is done where latency is all there is
+// (up to kSplitTokens) and every longer call keeps the one chain.
 RouterSplit router_split(int T, int E, int sms) {
   const int mt = (T + 127) / 128;
-  RouterSplit best{16, 1, false};
+  const bool split = T <= kSplitTokens;
+  RouterSplit best{16, 1, split};
   double cost = 1e30;
   for (int ch = 16; ch <= 128 && E % ch == 0; ch *= 2)
-    for (int ks = 1; ks <= 4; ks *= 2) {
+    for (int ks = 1; ks <= (split ? 4 : 1); ks *= 2) {
       const int waves = (int)(((long long)mt * (E / ch) * ks + sms - 1) / sms);
       const double c = waves * (6.0 + 32.0 / ks * (0.25 + ch * 0.002)) + 0.5 * ks;
       if (c < cost) {
@@ -605,7 +616,6 @@ RouterSplit router_split(int T, int E, int sms) {
         best.ksplit = ks;
       }
     }
-  best.stack = T <= kStackTokens;
   return best;
 }
 

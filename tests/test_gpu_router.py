@@ -14,9 +14,12 @@ from paper_2608_23805_gb300 import api
 
 pytestmark = pytest.mark.gpu
 
-# fp32-exact products, fp32 accumulation over H <= 2048 terms of size ~1: the
-# logits are within 1e-5 of fp64, the weights too; closer pairs may swap.
-TOL = 1e-5
+
+def tolerance(logits, H):
+    """The products are exact; each of a logit's 3 H / 16 accumulations drops at
+    most one unit in the last place (2^-23) of the running sum.  Four times
+    their random sum, at the largest logit; closer pairs may swap."""
+    return 4 * 2.0 ** -23 * (3 * H / 16) ** 0.5 * max(1.0, np.abs(logits).max())
 
 
 def route(x, wr, E, k, H, shared=False):
@@ -43,14 +46,15 @@ def check(x, wr, k, got):
     top = np.take_along_axis(logits, order, 1)
     n = min(k + 1, E)
     d = top[:, :n - 1] - top[:, 1:n] if n > 1 else np.ones((len(top), 1))
-    clear = ((d == 0) | (d > 2 * TOL)).all(axis=1)
-    assert clear.mean() > 0.95
+    tol = tolerance(logits, x.shape[1])
+    clear = ((d == 0) | (d > 2 * tol)).all(axis=1)
+    assert clear.mean() >= 0.7  # most rows decide the order
     assert (ids[clear] == order[clear, :k]).all()
     e = np.exp(top[:, :k] - top[:, :1])
-    assert np.abs(w - e / e.sum(1, keepdims=True)).max() <= TOL
+    assert np.abs(w - e / e.sum(1, keepdims=True)).max() <= tol
     assert (counts == np.bincount(ids.ravel(), minlength=E)).all()
     if k < E:
-        assert np.abs(gap - (top[:, k - 1] - top[:, k])).max() <= 2 * TOL
+        assert np.abs(gap - (top[:, k - 1] - top[:, k])).max() <= 2 * tol
     else:
         assert np.isinf(gap).all()
 
