@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1)
     const int r0 = gt >> 3;               // rows r0 + 16 i
     uint32_t it = 0;
     bool ok = true;
-    // permuted-row entries (t*k + j, or -1 past the expert's segment) of this
+    // permuted-row entries (a token, or -1 past the expert's segment) of this
     // thread's eight rows, loaded one tile ahead so that the next tile's first
     // copies do not wait on the group and permutation loads
     auto tile_rows = [&](int t, int (&pr)[8]) {
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(Cfg<MODE>::kThreads, 1)
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         if (pr[i] >= 0) {
-          src[i] = a.x + (size_t)(pr[i] / a.top_k) * a.x_ld + chunk * 8;
+          src[i] = a.x + (size_t)pr[i] * a.x_ld + chunk * 8;
           nbytes[i] = 16;
         } else {
           src[i] = a.x;

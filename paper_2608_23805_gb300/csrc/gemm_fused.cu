@@ -294,8 +294,8 @@ __global__ void __launch_bounds__(kFThreads, 1)
     const int r0 = gt >> 3;                           // rows r0 + 16 i
     uint32_t it = 0;
     bool ok = true;
-    // this thread's eight permutation entries of gate-up tile t (routed row
-    // token * k + j; -1 past the group's segment), loaded one tile ahead and
+    // this thread's eight permutation entries of gate-up tile t (a
+    // token; -1 past the group's segment), loaded one tile ahead and
     // first used at that tile's start, so the loads' latency is not waited
     // for at the start of the current tile
     auto tile_rows = [&](int t, int (&pr)[8]) {
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           if (pr[i] >= 0) {
-            src[i] = a.x + (size_t)(pr[i] / a.top_k) * a.x_ld + chunk * 8;
+            src[i] = a.x + (size_t)pr[i] * a.x_ld + chunk * 8;
             nbytes[i] = 16;
           } else {
             src[i] = a.x;

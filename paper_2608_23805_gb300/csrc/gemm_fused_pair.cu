@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(QCfg<Q4>::kThreads, 1)
     uint32_t it = 0;
     bool ok = true;
     // this thread's eight A rows of tile t: a gate-up tile's permutation
-    // entries (token * k + j), a down tile's h rows; -1 past the group's
+    // entries (tokens), a down tile's h rows; -1 past the group's
     // segment.  Loaded one tile ahead and first used at that tile's start.
     auto tile_rows = [&](int t, int (&pr)[8]) {
       const QTile tc = qdecode(a, ng, s_pt, t);
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(QCfg<Q4>::kThreads, 1)
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         if (pr[i] >= 0) {
-          src[i] = src_base + (size_t)(tc.up ? pr[i] / a.top_k : pr[i]) * ld + chunk * 8;
+          src[i] = src_base + (size_t)pr[i] * ld + chunk * 8;
           nbytes[i] = 16;
         } else {
           src[i] = src_base;

@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(PCfg<MODE>::kThreads, 1)
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         if (pr[i] >= 0) {
-          src[i] = a.x + (size_t)(pr[i] / a.top_k) * a.x_ld + chunk * 8;
+          src[i] = a.x + (size_t)pr[i] * a.x_ld + chunk * 8;
           nbytes[i] = 16;
         } else {
           src[i] = a.x;

@@ -86,8 +86,7 @@ struct GemmArgs {
   __nv_bfloat16* out;
   const __nv_bfloat16* x;   // gather source rows [T, H]
   int x_ld;
-  const int* perm;          // permuted row -> t*k + j
-  int top_k;
+  const int* perm;          // permuted row -> token
   int* status;
   long long wait_limit;     // clock64 cycles per bounded wait
   // non-zero: the epilogue's first thread also waits on a barrier nothing
@@ -132,8 +131,7 @@ struct FusedArgs {
   int y_ld;
   const __nv_bfloat16* x;   // [T, H]
   int x_ld;
-  const int* perm;          // permuted row -> t k + j
-  int top_k;
+  const int* perm;          // permuted row -> token
   int* ready;               // [m-tiles] finished gate-up tiles per 128-row tile (zero at launch)
   int* status;
   long long wait_limit;
@@ -160,6 +158,14 @@ struct FusedArgs {
   int q13_scale_ld;               // bytes of scales per W13 row (H / 16)
   long long q2_scale_off;         // byte offset of the W2 scales in an extent
   int q2_scale_ld;                // bytes of scales per W2 row (I / 16)
+  // gemm_cols.cu: the shared expert as one more group (sh_rows = T; 0: none),
+  // its weight block and intermediates, and the rings (cols_rings)
+  int sh_rows, sh_slot;
+  __nv_bfloat16* hs;              // [T, I]
+  __nv_bfloat16* ys;              // [T, H]
+  int tile_tok;                   // tokens per tile (32, 64 or 128)
+  int b_rows;                     // token rows per step in a stage (16 .. 128)
+  int ring_s, ring_w;             // stages; 4-bit: code slots (both powers of two)
 };
 
 // ---------------------------------------------------------------------------
@@ -182,6 +188,16 @@ cudaError_t launch_fused_wave_pair(const CUtensorMap& tmW13, const CUtensorMap& 
 // 4-bit waves on CTA pairs (tmQ13 / tmQ2: the byte-granular code maps).
 cudaError_t launch_fused_wave_pair_q4(const CUtensorMap& tmQ13, const CUtensorMap& tmQ2,
                                       const FusedArgs& a, const WaveParams& w, int max_pairs, cudaStream_t s);
+
+// Weights as MMA rows, tokens as columns (gemm_cols.cu): both projections and
+// the shared expert in one cooperative launch.  tmW13 / tmS13: gate and
+// up rows in pairs (bf16), 64-row boxes (4-bit); tmW2 / tmS2: 128-row boxes.
+// The shared expert's maps are of bf16 rows in both.
+int cols_tile_tokens(long long rows, int groups);
+void cols_rings(FusedArgs& a, bool q4, int T);
+cudaError_t launch_fused_cols(bool q4, const CUtensorMap& tmW13, const CUtensorMap& tmW2, const CUtensorMap& tmS13,
+                              const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid,
+                              cudaStream_t s);
 
 // GEMM tiling
 constexpr int kBM = 128;
@@ -259,6 +275,96 @@ struct FusedSched {
   }
 };
 
+struct ColsTile {
+  int up, g, m, n;
+};
+
+// Schedule of gemm_cols.cu over `ng` routed groups (token-tile prefix mt[]) and
+// a shared group (index ng) of mt_sh token tiles.  The up tiles are one
+// sequence with the shared group's spread evenly through it, the down tiles
+// another; a CTA takes a contiguous part of the up tiles, then the down tiles
+// that make up for one up tile fewer (a tile being worth w of them), then a
+// part of the rest.  Within a part: a run of the shared group's tiles and one
+// of the routed tiles, each walked token tile first, then weight rows, then
+// group.
+struct ColsWalk {
+  const int* mt;
+  int ng, mt_sh, nt_up, nt_dn;
+  int end[6];  // parts: [end[0], end[1]) up, [end[2], end[3]) and [end[4], end[5]) down
+  int run, left;
+  ColsTile t;
+
+  __host__ __device__ __forceinline__ void init(const int* s_mt, int ng_, int mt_sh_, int nt_up_, int nt_dn_, int P,
+                                                int c, int w) {
+    mt = s_mt;
+    ng = ng_;
+    mt_sh = mt_sh_;
+    nt_up = nt_up_;
+    nt_dn = nt_dn_;
+    const int U = (mt[ng] + mt_sh) * nt_up, D = (mt[ng] + mt_sh) * nt_dn;
+    const int hi = U % P, lo = P - hi;
+    end[0] = c * (U / P) + (c < hi ? c : hi);
+    end[1] = end[0] + U / P + (c < hi);
+    const int DA = hi > 0 ? (D < w * lo ? D : w * lo) : 0;
+    const int ca = c > hi ? c - hi : 0;
+    end[2] = (int)((long long)ca * DA / lo);
+    end[3] = c >= hi ? (int)((long long)(ca + 1) * DA / lo) : end[2];
+    const int DB = D - DA;
+    end[4] = DA + (int)((long long)c * DB / P);
+    end[5] = DA + (int)((long long)(c + 1) * DB / P);
+    run = -1;
+    left = 0;
+  }
+  // shared tiles among the first p of the sequence
+  __host__ __device__ __forceinline__ int shared_before(int p, int nt) const {
+    return mt_sh == 0 ? 0 : (int)((long long)p * (mt_sh * nt) / ((long long)(mt[ng] + mt_sh) * nt));
+  }
+  // to the next tile; false at the end
+  __host__ __device__ __forceinline__ bool next() {
+    if (left > 0) {
+      --left;
+      const int gm = t.g == ng ? mt_sh : mt[t.g + 1] - mt[t.g];
+      if (++t.m == gm) {
+        t.m = 0;
+        if (++t.n == (t.up ? nt_up : nt_dn)) {
+          t.n = 0;
+          ++t.g;  // every routed group has a tile
+        }
+      }
+      return true;
+    }
+    while (++run < 6) {
+      const int part = run >> 1;
+      const bool sh = (run & 1) == 0;
+      const int p0 = part == 0 ? end[0] : part == 1 ? end[2] : end[4];
+      const int p1 = part == 0 ? end[1] : part == 1 ? end[3] : end[5];
+      const int nt = part == 0 ? nt_up : nt_dn;
+      const int f0 = shared_before(p0, nt), f1 = shared_before(p1, nt);
+      const int tt = sh ? f0 : p0 - f0;
+      left = (sh ? f1 : p1 - f1) - tt;
+      if (left == 0) continue;
+      --left;
+      t.up = part == 0;
+      int lo = ng, base = 0, gm = mt_sh;
+      if (!sh) {
+        lo = 0;
+        int hi = ng - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (mt[mid] * nt <= tt) lo = mid; else hi = mid - 1;
+        }
+        base = mt[lo] * nt;
+        gm = mt[lo + 1] - mt[lo];
+      }
+      t.g = lo;
+      t.n = (tt - base) / gm;
+      t.m = (tt - base) - t.n * gm;
+      return true;
+    }
+    return false;
+  }
+};
+
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
@@ -328,6 +434,9 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t 
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
                "r"(src_bytes)
                : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");

@@ -134,7 +134,7 @@ struct SetupArgs {
   Group* groups;
   int* total_mtiles;   // [0]: 128-row tiles, [1]: 256-row pair tiles
   int* status;
-  int* ready;          // fused wave: per-m-tile counters, zeroed here (or nullptr)
+  int* ready;          // the next wave's tile counters, zeroed here (or nullptr)
   int n_ready;
 };
 

@@ -3,7 +3,7 @@
 // generation publication, and the weighted combine.
 //
 // Permutation: row r in [offsets[e], offsets[e+1]) holds the (t, j) pairs
-// routed to expert e in (t, j) order; perm[r] = t*k + j, inv[t*k + j] = r.
+// routed to expert e in (t, j) order; perm[r] = t, inv[t*k + j] = r.
 // Atomic-free: per-router-block counts (written by the router kernel) ->
 // column prefix over blocks -> per-warp stable ranks from __match_any_sync.
 //
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kScatterWarps * 32) scatter_kernel(const Scatt
       if (valid) {
         before = run[warp][e];
         const int pos = offs[e] + pre[j] + before + __popc(mask & lt);
-        a.perm[pos] = f;
+        a.perm[pos] = f / a.k;
         a.inv[f] = pos;
       }
       __syncwarp();

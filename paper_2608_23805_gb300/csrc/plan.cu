@@ -119,6 +119,34 @@ bool make_tmap_codes(CUtensorMap* m, const void* base, uint64_t row_bytes, uint6
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Boxes of 128 swizzled bytes (256 codes) x box_rows over packed 4-bit codes.
+bool make_tmap_codes128(CUtensorMap* m, const void* base, uint64_t row_bytes, uint64_t rows, uint32_t box_rows) {
+  auto fn = encode_fn();
+  if (fn == nullptr || rows == 0) return false;
+  cuuint64_t dims[2] = {row_bytes, rows};
+  cuuint64_t strides[1] = {row_bytes};
+  cuuint32_t box[2] = {128, box_rows};
+  cuuint32_t es[2] = {1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// bf16 rows [rows, H] as [H, 16 rows, rows / 16, +0 / +I rows]: a box lands as
+// 16 gate rows, then the same units' 16 up rows (I rows on), 128 swizzled bytes
+// each.  W13 blocks start on a multiple of 16 rows.
+bool make_tmap_pairs(CUtensorMap* m, const void* base, uint64_t H, uint64_t I, uint64_t rows) {
+  auto fn = encode_fn();
+  if (fn == nullptr || rows <= I) return false;
+  cuuint64_t dims[4] = {H, 16, (rows - I) / 16, 2};
+  cuuint64_t strides[3] = {2 * H, 32 * H, 2 * H * I};
+  cuuint32_t box[4] = {64, 16, 1, 2};
+  cuuint32_t es[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Reference-counted pool of CUDA events (readiness and consumer fences).
 struct EventPool {
   std::vector<cudaEvent_t> ev;
@@ -240,6 +268,10 @@ struct msi_plan {
   int fwd_ev = -1;
   CUtensorMap tm_w13{}, tm_w2{}, tm_sh13{}, tm_sh2{};
   CUtensorMap tm_q13{}, tm_q2{};  // 4-bit plans: packed codes of W13 / W2 over the pool
+  // gemm_cols.cu: W13 of the pool and of the shared expert (bf16 plans: gate
+  // and up rows in pairs; 4-bit plans: 64-row boxes of codes, of bf16 rows),
+  // and the 4-bit plans' W2 codes
+  CUtensorMap tm_p13{}, tm_psh13{}, tm_c2{};
   std::vector<msi_trace_rec> trace;
   uint64_t seq = 0;
   msi_counters ctr{};
@@ -358,7 +390,8 @@ WsLayout layout(const msi_plan* p, int T) {
   L.yp = take(2 * Tk * H);
   // fused GEMMs: a counter per 128-row tile, two banks (consecutive waves
   // alternate; each wave's kernel zeroes the other bank for the next)
-  L.ready_n = Tk / kBM + E + 1;
+  const size_t tile = cols_tile_tokens((long long)Tk, (int)E);
+  L.ready_n = Tk / tile + E + 1 + (p->d.has_shared ? (size_t)T / tile + 1 : 0);
   L.ready = take(2 * 4 * L.ready_n);
   if (p->d.has_shared) {
     L.hs = take(2 * (size_t)T * I);
@@ -702,6 +735,22 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
   return MSI_OK;
 }
 
+// Weights as MMA rows (gemm_cols.cu), in one launch with a resident call's
+// shared expert, while the groups average fewer rows than a tile holds:
+//   4-bit (one conversion per weight and tile): at 8, 250 and 4,096 tokens of
+//     the Qwen-shaped layer 70, 328 and 520 us against 91, 534 and 546 in two
+//     row-major launches; more than 128 rows take two tiles, two conversions;
+//   bf16: where the launches' latency is what counts (one token: 24 us for
+//     what took 28 + 25 on a side stream); from some 40 tokens on both
+//     orientations stream the weights at the same rate (0.97 of HBM), and the
+//     row-major tiles read the tokens half as often.  Not a wave: its launch
+//     has no shared expert to take in.
+constexpr long long kColsMaxRows = 128, kColsMaxRowsBf16 = 8;
+bool cols_tiles(const msi_plan* p, const FwdCtx& f, long long rows, int ng, bool wave = false) {
+  return !(f.flags & (MSI_FWD_SPLIT_WAVES | MSI_FWD_SINGLE_CTA)) && ng > 0 && rows < kColsMaxRows * ng &&
+         (p->d.wdtype == MSI_W_Q4G32 || (!wave && rows < kColsMaxRowsBf16 * ng));
+}
+
 // Router + histogram over the call's rows for router weight `rw`: the route
 // event (ids, weights, gap) and per-expert counts go to `ev`.  first: the
 // forward's own routing (its first kernel clears the status word and writes
@@ -766,7 +815,7 @@ msi_status route_rows(msi_plan* p, FwdCtx& f, const float* rw, const msi_route_e
     const bool fuse = first && xa != nullptr && f.T <= kFuseTokens;
     // a long resident call begins with a kernel of its own, so that the side
     // stream's shared expert runs beside the logits and not after them
-    const bool begun = first && tp.E > 0 && d.has_shared && f.T >= 4096;
+    const bool begun = first && tp.E > 0 && d.has_shared && f.T >= 4096 && !cols_tiles(p, f, (long long)f.T * k, E);
     if (begun) {
       LAUNCH(p, MSI_K_UPLOAD, s, launch_upload(tp, ra.tab_slot, ra.tab_expected, ra.status, ra.sh, ra.sh_total, s));
       CK(cudaEventRecord(p->ev_fork, s));
@@ -890,7 +939,7 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
     xa.tab_slot = at<int>(ws, L.table);
     xa.tab_expected = at<unsigned long long>(ws, L.expected);
     xa.layer = tp.layer;
-    if (fused_resident(p, f, (long long)f.T * k, E)) {
+    if (fused_resident(p, f, (long long)f.T * k, E) || cols_tiles(p, f, (long long)f.T * k, E)) {
       xa.ready = at<int>(ws, L.ready);
       xa.n_ready = ready_bank(f);
     }
@@ -935,7 +984,6 @@ GemmArgs gateup_args(msi_plan* p, FwdCtx& f, const Group* groups, int ng, const 
   g.x = static_cast<const __nv_bfloat16*>(f.x);
   g.x_ld = d.hidden;
   g.perm = at<int>(f.ws, f.L.perm);
-  g.top_k = d.top_k;
   g.status = at<int>(f.ws, f.L.status);
   g.wait_limit = p->wait_cycles;
   g.stall = f.stall;
@@ -995,7 +1043,8 @@ msi_status routed_ffn(msi_plan* p, FwdCtx& f, int ng, int grid1, int grid2, long
   const int q13_rows = (int)(d.extent_bytes / (d.hidden / 2));
   const int q2_rows = (int)(d.extent_bytes / (d.inter / 2));
   const int q2_off = (int)(HI / (d.inter / 2));
-  if (wave_mtiles >= 0 && fused_wave(p, f, rows, ng)) {
+  const bool cols = wave_mtiles >= 0 && cols_tiles(p, f, rows, ng, wp != nullptr);
+  if (cols || (wave_mtiles >= 0 && fused_wave(p, f, rows, ng))) {
     // one launch: the wave's gate-up tiles, then its down tiles
     FusedArgs fa{};
     fa.groups = groups;
@@ -1017,7 +1066,6 @@ msi_status routed_ffn(msi_plan* p, FwdCtx& f, int ng, int grid1, int grid2, long
     fa.x = static_cast<const __nv_bfloat16*>(f.x);
     fa.x_ld = d.hidden;
     fa.perm = at<int>(f.ws, f.L.perm);
-    fa.top_k = d.top_k;
     int* bank0 = at<int>(f.ws, f.L.ready);
     int* bank1 = bank0 + f.L.ready_n;
     fa.ready = (wave & 1) ? bank1 : bank0;
@@ -1045,7 +1093,6 @@ msi_status routed_ffn(msi_plan* p, FwdCtx& f, int ng, int grid1, int grid2, long
     const int spare = wp != nullptr ? 1 : 0;
     const int pairs = (int)std::min<long long>(p->sms / 2 - spare, std::max<long long>(1, tiles));
     if (!bf16) {
-      // 4-bit waves: CTA pairs (fused_wave admits them from 512 rows per group)
       fa.q4_pool = static_cast<const uint8_t*>(d.slot_pool);
       fa.q4_extent = d.extent_bytes;
       fa.q13_rows_per_slot = q13_rows;
@@ -1055,6 +1102,28 @@ msi_status routed_ffn(msi_plan* p, FwdCtx& f, int ng, int grid1, int grid2, long
       fa.q13_scale_ld = d.hidden / 16;
       fa.q2_scale_off = 3 * HI / 2 + HI / 8;
       fa.q2_scale_ld = d.inter / 16;
+    }
+    if (cols) {
+      fa.tile_tok = std::max(cols_tile_tokens(rows, ng), cols_tile_tokens((long long)f.T * d.top_k, d.n_experts));
+      fa.nt_up = d.inter / 64;
+      fa.nt_dn = d.hidden / 128;
+      long long all = (long long)wave_mtiles * (fa.nt_up + fa.nt_dn);
+      if (wp == nullptr && d.has_shared) {
+        fa.sh_rows = f.T;
+        fa.sh_slot = f.layer;
+        fa.hs = at<__nv_bfloat16>(f.ws, f.L.hs);
+        fa.ys = at<__nv_bfloat16>(f.ws, f.L.ys);
+        all += (long long)((f.T + fa.tile_tok - 1) / fa.tile_tok) * (fa.nt_up + fa.nt_dn);
+      }
+      cols_rings(fa, !bf16, f.T);
+      const int grid = (int)std::min<long long>(p->sms - spare, std::max<long long>(1, all));
+      LAUNCH(p, MSI_K_FFN, f.cs,
+             launch_fused_cols(!bf16, p->tm_p13, bf16 ? p->tm_w2 : p->tm_c2, d.has_shared ? p->tm_psh13 : p->tm_p13,
+                               d.has_shared ? p->tm_sh2 : p->tm_p13, fa, wv, grid, f.cs));
+      return MSI_OK;
+    }
+    if (!bf16) {
+      // 4-bit waves: CTA pairs (fused_wave admits them from 512 rows per group)
       LAUNCH(p, MSI_K_FFN, f.cs, launch_fused_wave_pair_q4(p->tm_q13, p->tm_q2, fa, wv, pairs, f.cs));
       return MSI_OK;
     }
@@ -1273,18 +1342,23 @@ msi_status msi_plan_create(const msi_plan_desc* desc, msi_plan** out) {
   const uint64_t H = d.hidden, I = d.inter, S = d.n_slots;
   if (d.wdtype == MSI_W_BF16) {
     if (!make_tmap(&p->tm_w13, d.slot_pool, H, S * 3 * I, 128) ||
-        !make_tmap(&p->tm_w2, d.slot_pool, I, S * 3 * H, 128))
+        !make_tmap(&p->tm_w2, d.slot_pool, I, S * 3 * H, 128) ||
+        !make_tmap_pairs(&p->tm_p13, d.slot_pool, H, I, S * 3 * I))
       return fail(MSI_ERR_CUDA);
   }
   if (d.wdtype == MSI_W_Q4G32) {
     if (d.extent_bytes % (H / 2) || d.extent_bytes % (I / 2) ||
         !make_tmap_codes(&p->tm_q13, d.slot_pool, H / 2, S * (d.extent_bytes / (H / 2))) ||
-        !make_tmap_codes(&p->tm_q2, d.slot_pool, I / 2, S * (d.extent_bytes / (I / 2))))
+        !make_tmap_codes(&p->tm_q2, d.slot_pool, I / 2, S * (d.extent_bytes / (I / 2))) ||
+        !make_tmap_codes128(&p->tm_p13, d.slot_pool, H / 2, S * (d.extent_bytes / (H / 2)), 64) ||
+        !make_tmap_codes128(&p->tm_c2, d.slot_pool, I / 2, S * (d.extent_bytes / (I / 2)), 128))
       return fail(MSI_ERR_CUDA);
   }
   if (d.has_shared) {
     if (!make_tmap(&p->tm_sh13, d.shared_w, H, (uint64_t)d.n_layers * 3 * I, 128) ||
-        !make_tmap(&p->tm_sh2, d.shared_w, I, (uint64_t)d.n_layers * 3 * H, 128))
+        !make_tmap(&p->tm_sh2, d.shared_w, I, (uint64_t)d.n_layers * 3 * H, 128) ||
+        !(d.wdtype == MSI_W_BF16 ? make_tmap_pairs(&p->tm_psh13, d.shared_w, H, I, (uint64_t)d.n_layers * 3 * I)
+                                 : make_tmap(&p->tm_psh13, d.shared_w, H, (uint64_t)d.n_layers * 3 * I, 64)))
       return fail(MSI_ERR_CUDA);
   }
   *out = p;
@@ -1479,7 +1553,8 @@ msi_status forward_resident(msi_plan* p, int layer, const void* x, int T, const 
   }
   st = front(p, f, tp);
   if (st != MSI_OK) return st;
-  const bool fork = d.has_shared && T > 0;
+  const bool cols = cols_tiles(p, f, (long long)T * d.top_k, E);
+  const bool fork = d.has_shared && T > 0 && !cols;
   if (fork) {
     // the shared expert needs no routing: it runs on the side stream while
     // the router, scan and scatter leave most SMs idle, and joins before the
@@ -1496,7 +1571,7 @@ msi_status forward_resident(msi_plan* p, int layer, const void* x, int T, const 
     const int g1 = (int)std::min<long long>(p->sms, mt_max * (d.inter / 128));
     const int g2 = (int)std::min<long long>(p->sms, mt_max * (d.hidden / kBN));
     st = routed_ffn(p, f, E, g1, g2, (long long)T * d.top_k,
-                    fused_resident(p, f, (long long)T * d.top_k, E) ? (int)mt_max : -1);
+                    cols || fused_resident(p, f, (long long)T * d.top_k, E) ? (int)mt_max : -1);
     if (st != MSI_OK) return st;
     st = consumer_record(p, used, f.cs);
     if (st != MSI_OK) return st;
@@ -1853,7 +1928,7 @@ msi_status forward_streamed(msi_plan* p, int layer, const void* x, int T, const 
     }
     st = wait_ready(p, used, f.cs);
     if (st != MSI_OK) return st;
-    const bool fused = fused_wave(p, f, wave_rows, wp.n);
+    const bool fused = fused_wave(p, f, wave_rows, wp.n) || cols_tiles(p, f, wave_rows, wp.n, true);
     if (!fused) {
       // split launches: the setup kernel re-checks the wave's slots and
       // builds its groups (a fused wave's kernel does both itself)
@@ -1866,6 +1941,9 @@ msi_status forward_streamed(msi_plan* p, int layer, const void* x, int T, const 
       sa.groups = at<Group>(ws, f.L.groups);
       sa.total_mtiles = at<int>(ws, f.L.total);
       sa.status = at<int>(ws, f.L.status);
+      // the next wave may run in one launch: its bank of tile counters
+      sa.ready = at<int>(ws, f.L.ready) + ((w & 1) ? 0 : f.L.ready_n);
+      sa.n_ready = (int)f.L.ready_n;
       LAUNCH(p, MSI_K_SETUP, f.cs, launch_setup_wave(sa, wp, f.cs));
     }
     const int g1 = std::max(1, std::min(p->sms, mtiles * (d.inter / 128)));

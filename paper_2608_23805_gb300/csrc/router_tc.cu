@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(512, 2) router_select_scatter_kernel(const Rou
     const int tok = f / a.k, id = __ldcg(&a.ids[f]), w = tok >> 5;
     int pos = offs[id] + __popc(mask[w][id] & ((1u << (tok & 31)) - 1u));  // + the expert's earlier tokens
     for (int q = 0; q < w; ++q) pos += __popc(mask[q][id]);
-    s.perm[pos] = f;
+    s.perm[pos] = tok;
     s.inv[f] = pos;
   }
   if (s.tab_slot != nullptr) build_groups(s, e, cnt, base, slot, cnt > 0 ? code : 0, tmp);

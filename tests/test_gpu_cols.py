@@ -1,0 +1,65 @@
+"""The weights-as-rows FFN kernel (csrc/gemm_cols.cu): resident and streamed
+calls at the edges of its tiles, against the fp64 oracle, and against the
+row-major split launches of the same call.
+
+Shapes: tiles of 1 to 128 tokens and several per expert, H and I whose 4-bit
+code rows end inside a weight slot, groups without rows, with and without the
+shared expert (its group's tiles are bf16 in both weight formats)."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from gpu_case import Case, bf16_bits, bf16_tensor, compare_out, compare_routes
+
+pytestmark = pytest.mark.gpu
+
+
+def run_case(tokens, wdtype, streamed, hidden, inter, experts, top_k, shared, residual=False):
+    cfg = synth.config("tiny", hidden=hidden, inter=inter, n_experts=experts, top_k=top_k, tokens=tokens,
+                       n_slots=8 if streamed else experts, wdtype=wdtype, has_shared=shared)
+    case = Case(cfg)
+    x_bits = synth.hidden(cfg)
+    x = bf16_tensor(x_bits)
+    ref = case.oracle_layer(x_bits, residual=residual)
+    if streamed:
+        out, ev = case.plan.forward_streamed(0, x, case.router[0], residual=residual)
+    else:
+        table, gens = case.stage_all()
+        out, ev = case.plan.forward(0, x, case.router[0], table, gens, residual=residual)
+        split, _ = case.plan.forward(0, x, case.router[0], table, gens, residual=residual, single_cta=True,
+                                     split_waves=True)
+    torch.cuda.synchronize()
+    assert case.plan.status() == 0
+    compare_routes(ev.ids.cpu().numpy(), ev.weights.cpu().numpy(), ref)
+    compare_out(bf16_bits(out), ref["out"])
+    if not streamed:
+        # the same products summed in fp32 over the same K order: outputs
+        # differ by no more than a rounding of h and of y
+        a, b = out.float(), split.float()
+        assert (a - b).norm() <= 2e-3 * b.norm()
+    case.close()
+
+
+@pytest.mark.parametrize("tokens", [1, 2, 15, 17, 33, 64, 129, 500, 700])
+@pytest.mark.parametrize("streamed", [False, True])
+def test_q4_lengths(tokens, streamed):
+    run_case(tokens, synth.W_Q4G32, streamed, 512, 256, 16, 4, not streamed)
+
+
+@pytest.mark.parametrize("hidden,inter,experts,top_k", [(256, 128, 16, 2), (768, 384, 8, 1), (1024, 640, 24, 8),
+                                                        (2048, 512, 64, 10)])
+@pytest.mark.parametrize("shared", [False, True])
+def test_q4_shapes(hidden, inter, experts, top_k, shared):
+    run_case(90, synth.W_Q4G32, False, hidden, inter, experts, top_k, shared, residual=True)
+
+
+@pytest.mark.parametrize("tokens", [1, 3, 16, 17, 40])
+@pytest.mark.parametrize("streamed", [False, True])
+def test_bf16_lengths(tokens, streamed):
+    run_case(tokens, synth.W_BF16, streamed, 512, 256, 64, 8, not streamed)
+
+
+@pytest.mark.parametrize("hidden,inter,experts,top_k", [(256, 128, 16, 2), (768, 384, 32, 1), (1024, 640, 64, 8)])
+def test_bf16_shapes(hidden, inter, experts, top_k):
+    run_case(20, synth.W_BF16, False, hidden, inter, experts, top_k, True)
