@@ -549,7 +549,11 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 // A value that every lane holds, as one the compiler can see to be uniform.
-__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_max_sync(0xffffffffu, v); }
+__device__ __forceinline__ uint32_t uniform(uint32_t v) {
+  uint32_t r;
+  asm volatile("redux.sync.max.u32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(v));
+  return r;
+}
 // A wait of the whole warp, with one answer.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                long long limit) {
