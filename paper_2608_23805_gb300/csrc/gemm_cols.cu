@@ -15,13 +15,15 @@
 //   down tile (g, m, n):  128 output features: y[rows, 128 n .. 128 n + 128)
 // The resident shared expert is one more group (all tokens, identity rows).
 //
-// K goes by stages of two steps of 64, one tcgen05.commit a stage.
+// K goes by stages of four steps of 64 (two where four would leave too few
+// stages), one tcgen05.commit a stage: the issuing and the token warp's
+// per-stage instructions, not the MMAs, bound short tiles.
 // Weights (operand A):
 //   bf16: TMA into the stage, read by the MMA from shared memory;
 //   4-bit: TMA brings 128 rows x 256 codes (16 KB) and cp.async their scales
 //       into a ring of their own; sixteen warps in four sets (set j: every
-//       fourth stage) convert 128 codes of a row per thread and write them to a
-//       TMEM operand ring of four stages, from which the MMA reads A.
+//       fourth half stage) convert 128 codes of a row per thread and write them
+//       to a TMEM operand ring of two stages, from which the MMA reads A.
 //       The weights thus cross shared memory once, as codes: converted in
 //       shared memory they would cost 4 x their bf16 size in shared-memory
 //       traffic, which bounds the row-major 4-bit kernel.
@@ -31,7 +33,7 @@
 // What bounds it: for 4-bit the instructions of the converting and the issuing
 // warps (an MMA of up to 96 columns takes 48 cycles), not HBM; for bf16 and few
 // tokens the latency of a tile's pass over K.  Resident Qwen-shaped layer, both
-// projections: 4-bit 250 tokens 328 us (534 as two row-major launches), 8
+// projections: 4-bit 250 tokens 308 us (534 as two row-major launches), 8
 // tokens 70 us (91), 4,096 tokens 520 us (546); bf16 one token 24 us with the
 // shared expert (28 without it, which took 25 beside it).
 //
@@ -56,43 +58,22 @@ namespace {
 constexpr int kCSlot = 128 * 128;     // weight ring slot
 constexpr int kCScale = 128 * 16;     // 4-bit: its rows' eight scales
 constexpr int kCRingMax = 8;
-constexpr int STEPS = 2;              // 64-K steps per stage (K is a multiple of 128)
-constexpr int kCOperand = 4;          // 4-bit: stages that the TMEM operand ring holds
+constexpr int kCOperand = 4;          // 4-bit: half stages that the TMEM operand ring holds
 constexpr int kCTokWarps = 4;
 constexpr int kCDqWarp0 = 10;
 constexpr int kCDqWarps = 16;
 constexpr int kCTable = kMaxExperts + 1;  // groups: experts and the shared one
 
-template <bool Q4>
+template <bool Q4, int STEPS>
 struct CCfg {
   static constexpr int kThreads = (kCDqWarp0 + (Q4 ? kCDqWarps : 0)) * 32;
   static constexpr uint32_t kOperandCol = 256;  // TMEM: two accumulators of 128 columns, then A steps
 };
 
-// mbar_wait that sleeps NS nanoseconds between polls (0: none).  A waiting
-// warp's polls take issue slots from the converting ones: without the sleep
-// they were over half of the 4-bit kernel's instructions (1,468 per scheduler
-// and 256 of K).
-template <int NS>
-__device__ __forceinline__ bool cwait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (clock64() - t0 > limit) {
-      *abort_flag = 1;
-      return false;
-    }
-    if (NS > 0) __nanosleep(NS);
-  }
-}
-
-// By a whole warp, which is converged after it (what follows may be an aligned
-// TMEM access), with one answer.
-template <int NS>
-__device__ __forceinline__ bool cwait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
-  return __all_sync(0xffffffffu, cwait<NS>(bar, parity, abort_flag, limit));
+// mbar_wait by a whole warp, which is converged after it (what follows may be
+// an aligned TMEM access), with one answer.
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit));
 }
 
 // Ring position: slot index and the parity of its round.
@@ -160,8 +141,10 @@ __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
   return d;
 }
 
-// dequant8 on the FMA pipe: eight 4-bit codes -> eight bf16 weights s (q - 8),
-// each rounded once, in packed bf16 arithmetic.  A code as the low bits of a
+// Eight 4-bit codes -> eight bf16 weights s (q - 8), each rounded once (the
+// bits of dequant8), in packed bf16 arithmetic: 33 cycles a word and scheduler
+// against 36, and seven instead of fifteen on the ALU pipe that the rest of
+// the kernel needs (250 tokens: 308 us, with dequant8 318).  A code as the low bits of a
 // bf16 is the subnormal q 2^-133; one FMA makes it (q - 8) / 64 exactly.  64 s
 // (11 bits) = hi + lo exactly with hi = bf16(64 s); (q - 8) / 64 * lo is exact
 // (4 + 4 bits), and the last FMA adds the exact product with hi and rounds.
@@ -181,20 +164,8 @@ __device__ __forceinline__ uint4 dequant8_bf16(uint32_t w, uint32_t hi, uint32_t
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// 32 codes of a row under one fp16 scale -> 16 TMEM columns of the thread's
-// lane, by either conversion (the same bits).  The groups of 32 alternate
-// between them: dequant8 is bound by the ALU pipe (36 cycles a word and
-// scheduler), the bf16 one by the FMA pipe (33), so that both work.
+// 32 codes of a row under one fp16 scale -> 16 TMEM columns of the thread's lane.
 __device__ __forceinline__ void convert32(const uint4& c, uint32_t scale, uint32_t dst) {
-  const float s = __half2float(__ushort_as_half((unsigned short)scale));
-  const uint64_t s2 = f32x2(s, s), n2 = f32x2(-136.0f * s, -136.0f * s);
-  const uint4 a0 = dequant8(c.x, s2, n2), a1 = dequant8(c.y, s2, n2);
-  const uint4 a2 = dequant8(c.z, s2, n2), a3 = dequant8(c.w, s2, n2);
-  const uint32_t o[16] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w,
-                          a2.x, a2.y, a2.z, a2.w, a3.x, a3.y, a3.z, a3.w};
-  tmem_st16(dst, o);
-}
-__device__ __forceinline__ void convert32_bf16(const uint4& c, uint32_t scale, uint32_t dst) {
   const float s = 64.0f * __half2float(__ushort_as_half((unsigned short)scale));
   const uint32_t hi = pack_bf16x2(s, s);
   const float rest = s - bf16_lo(hi);
@@ -310,12 +281,12 @@ __device__ __forceinline__ int cols_group_table(const FusedArgs& a, const WavePa
 
 }  // namespace
 
-template <bool Q4>
-__global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
+template <bool Q4, int STEPS>
+__global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
     fused_cols_kernel(const __grid_constant__ CUtensorMap tmW13, const __grid_constant__ CUtensorMap tmW2,
                       const __grid_constant__ CUtensorMap tmS13, const __grid_constant__ CUtensorMap tmS2,
                       const __grid_constant__ FusedArgs a, const __grid_constant__ WaveParams w) {
-  using C = CCfg<Q4>;
+  using C = CCfg<Q4, STEPS>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -407,10 +378,11 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
           const int row = t.up ? slot * a.w13_rows_per_slot + t.n * 64
                                : slot * a.w2_rows_per_slot + a.w2_row_off + t.n * 128;
           for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-            if (!cwait<64>(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
-            mbar_arrive_expect_tx(&sfull[r.i], STEPS * kCSlot);
+            if (!mbar_wait(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+            const int k1 = min(kb_n, k0 + STEPS);
+            mbar_arrive_expect_tx(&sfull[r.i], (k1 - k0) * kCSlot);
             uint8_t* dst = sT + r.i * stage;
-            for (int kb = k0; kb < k0 + STEPS; ++kb, dst += kCSlot) {
+            for (int kb = k0; kb < k1; ++kb, dst += kCSlot) {
               if (!t.up) {
                 tma_load_2d(dst, map, &sfull[r.i], kb * 64, row);
               } else {
@@ -462,7 +434,7 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
           }
         }
         for (int s = 0; s < slots; ++s) {
-          if (!cwait<64>(&wempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+          if (!mbar_wait(&wempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
           if (lane == 0) {
             mbar_arrive_expect_tx(&wfull[r.i], kCSlot);
             uint8_t* dst = sW + r.i * kCSlot;
@@ -520,35 +492,58 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
       const int kb_n = (int)uniform(t.up ? a.kb_up : a.kb_dn);
       const uint32_t cols = uniform(min(a.tile_tok, s_cnt[t.g] - t.m * a.tile_tok));
       const uint32_t idesc = idesc_bf16(128, (cols + 15) & ~15);
-      ok = cwait_warp<0>(&tempty[acc], aph ^ 1, abort_flag, lim);
+      ok = wait_warp(&tempty[acc], aph ^ 1, abort_flag, lim);
       if (!ok) break;
       const uint32_t d = tm + acc * 128;
       for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-        ok = cwait_warp<0>(&sfull[r.i], r.ph, abort_flag, lim);
-        if (ok && Q4) ok = cwait_warp<0>(&afull[ra.i], ra.ph, abort_flag, lim);
+        ok = wait_warp(&sfull[r.i], r.ph, abort_flag, lim);
         if (!ok) break;
         // cp.async (generic proxy) wrote the tokens: before the tensor core's reads
         fence_proxy_async_smem();
-        tc_fence_after();
         const uint32_t w_lo = s_lo + ((r.i * stage) >> 4);
         const uint32_t bl = w_lo + (w_stage >> 4);
-        const uint32_t at = Q4 ? tm + C::kOperandCol + ra.i * (STEPS * 32) : w_lo;
-        if (elect_one()) {
+        if (Q4) {
+          // halves of two steps, as the conversion sets finish them (a stage
+          // past the tile's K has its second half announced empty)
 #pragma unroll
-          for (int j = 0; j < STEPS; ++j) {
-            const uint32_t bj = bl + j * (b_step >> 4);
+          for (int h = 0; h < 2; ++h) {
+            ok = wait_warp(&afull[ra.i], ra.ph, abort_flag, lim);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t at = tm + C::kOperandCol + ra.i * 64;
+            if (elect_one()) {
+              if (h == 0 || k0 + 2 < kb_n) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              if (Q4) umma_bf16_ts(d, at + 32 * j + 8 * k, desc64(bj + 2 * k, desc_hi), idesc, (k0 | j | k) != 0);
-              else umma_bf16(d, desc64(at + (kCSlot >> 4) * j + 2 * k, desc_hi), desc64(bj + 2 * k, desc_hi), idesc,
-                             (k0 | j | k) != 0);
+                for (int j = 0; j < 2; ++j) {
+                  const uint32_t bj = bl + (2 * h + j) * (b_step >> 4);
+#pragma unroll
+                  for (int k = 0; k < 4; ++k)
+                    umma_bf16_ts(d, at + 32 * j + 8 * k, desc64(bj + 2 * k, desc_hi), idesc, (k0 | h | j | k) != 0);
+                }
+              }
+              if (h == 1) umma_commit(&sempty[r.i]);
             }
+            __syncwarp();
+            ra.step();
           }
-          umma_commit(&sempty[r.i]);
+          if (!ok) break;
+        } else {
+          tc_fence_after();
+          if (elect_one()) {
+#pragma unroll
+            for (int j = 0; j < STEPS; ++j) {
+              if (j < 2 || k0 + j < kb_n) {
+                const uint32_t bj = bl + j * (b_step >> 4), wj = w_lo + j * (kCSlot >> 4);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  umma_bf16(d, desc64(wj + 2 * k, desc_hi), desc64(bj + 2 * k, desc_hi), idesc, (k0 | j | k) != 0);
+              }
+            }
+            umma_commit(&sempty[r.i]);
+          }
+          __syncwarp();
         }
-        __syncwarp();
         r.step();
-        ra.step();
       }
       if (!ok) break;
       if (elect_one()) umma_commit(&tfull[acc]);
@@ -567,7 +562,7 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
   } else if (warp < 4) {
     // ------------------------------------------------------------- epilogue
     uint32_t jt = 0;
-    if (a.stall && threadIdx.x == 0) cwait<200>(never, 0, abort_flag, lim);  // runs out: abort
+    if (a.stall && threadIdx.x == 0) mbar_wait(never, 0, abort_flag, lim);  // runs out: abort
     __syncwarp();
     while (walk.next()) {
       const ColsTile& t = walk.t;
@@ -575,7 +570,7 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
       const int row0 = t.m * a.tile_tok;
       const int rows = min(a.tile_tok, s_cnt[t.g] - row0);
       const uint32_t acc = jt & 1, aph = (jt >> 1) & 1;
-      if (!cwait_warp<200>(&tfull[acc], aph, abort_flag, lim)) break;
+      if (!wait_warp(&tfull[acc], aph, abort_flag, lim)) break;
       tc_fence_after();
       const uint32_t tb = tmem_base + ((uint32_t)(warp * 32) << 16) + acc * 128;
       const size_t orow = (size_t)(sh ? row0 : s_rb[t.g] + row0);
@@ -689,10 +684,14 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
         const uint32_t bytes = r0 < rows ? 16u : 0u;
         const __nv_bfloat16* src = r0 < rows ? base + (size_t)(t.up ? tok[0] : r0) * ld : a.x;
         for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-          if (!cwait<40>(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+          if (!mbar_wait(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
           const uint32_t dst = dst0 + r.i * stage;
           cp_async16_at(dst, src, bytes);
           cp_async16_at(dst + b_step, src + kBK, bytes);
+          if (STEPS == 4 && k0 + 2 < kb_n) {
+            cp_async16_at(dst + 2 * b_step, src + 2 * kBK, bytes);
+            cp_async16_at(dst + 3 * b_step, src + 3 * kBK, bytes);
+          }
           src += STEPS * kBK;
           cp_async_arrive_noinc(&sfull[r.i]);  // arrives when this thread's copies land
           r.step();
@@ -706,7 +705,7 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
         src[i] = r0 + 16 * i < rows ? base + (size_t)(t.up ? tok[i] : r0 + 16 * i) * ld : a.x;
       }
       for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-        if (!cwait<40>(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+        if (!mbar_wait(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
         const uint32_t dst = dst0 + r.i * stage;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -714,6 +713,10 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
           const uint32_t bytes = r0 + 16 * i < rows ? 16u : 0u;
           cp_async16_at(dst + i * 2048, src[i], bytes);
           cp_async16_at(dst + b_step + i * 2048, src[i] + kBK, bytes);
+          if (STEPS == 4 && k0 + 2 < kb_n) {
+            cp_async16_at(dst + 2 * b_step + i * 2048, src[i] + 2 * kBK, bytes);
+            cp_async16_at(dst + 3 * b_step + i * 2048, src[i] + 3 * kBK, bytes);
+          }
           src[i] += STEPS * kBK;
         }
         cp_async_arrive_noinc(&sfull[r.i]);
@@ -724,7 +727,10 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
   } else if (Q4) {
     // ------------------------------------------------------------- conversion
     const int q = warp & 3;                   // TMEM lane quarter
-    const int set = (warp - kCDqWarp0) >> 2;  // stages set, set + 4, ... of the CTA's sequence
+    // half stages set, set + 4, ... of the CTA's sequence: half set & 1 of the
+    // stages of parity set >> 1
+    const int set = (warp - kCDqWarp0) >> 2;
+    const uint32_t odd = set >> 1, half = set & 1;
     const uint32_t s_mask = a.ring_s - 1, s_log = 31 - __clz(a.ring_s);
     const uint32_t w_mask = a.ring_w - 1, w_log = 31 - __clz(a.ring_w);
     // the thread's row in a slot: down tiles in order, up tiles 64 gate rows,
@@ -739,53 +745,49 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
     while (ok && walk.next()) {
       const ColsTile& t = walk.t;
       const int kb_n = t.up ? a.kb_up : a.kb_dn;
-      const uint32_t n_st = kb_n / STEPS;
+      const uint32_t n_st = (kb_n + 3) / 4;
       const int at = t.up ? at_up : at_dn;
       const bool codes = t.g != g_sh;
+      // the stage that used this part of the TMEM ring (two before) has been consumed
+      auto stage_free = [&](uint32_t st) {
+        return st < 2 || wait_warp(&sempty[(st - 2) & s_mask], ((st - 2) >> s_log) & 1u, abort_flag, lim);
+      };
       if (codes) {
-        // the set's stages; a slot holds two, so a set passes over at most four
-        // slots between its own, no more than the ring has (a parity tells one
-        // round from the next)
-        for (uint32_t i = (set - st0) & 3u; i < n_st; i += 4) {
-          const uint32_t st = st0 + i;
-          const uint32_t wc = w0 + (i >> 1), wi = wc & w_mask;
-          if (!cwait_warp<20>(&wfull[wi], (wc >> w_log) & 1u, abort_flag, lim)) { ok = false; break; }
-          // the stage that used this part of the TMEM ring has been consumed
-          if (st >= kCOperand && !cwait_warp<20>(&sempty[(st - kCOperand) & s_mask], ((st - kCOperand) >> s_log) & 1u,
-                                            abort_flag, lim)) { ok = false; break; }
-          tc_fence_after();
-          // half a slot: 128 codes and four scales of the row
-          const uint32_t dst = tdst + set * (STEPS * 32);
-          const uint32_t src = sw0 + wi * kCSlot + at * 128 + (((i & 1u) << 6) ^ x0);
-          const uint2 sc = ld_shared_v2(ss0 + wi * kCScale + at * 16 + (i & 1u) * 8);
-          const uint4 c0 = ld_shared_v4(src + x[0]), c1 = ld_shared_v4(src + x[1]);
-          convert32(c0, sc.x & 0xFFFFu, dst);
-          const uint4 c2 = ld_shared_v4(src + x[2]);
-          convert32_bf16(c1, sc.x >> 16, dst + 16);
-          const uint4 c3 = ld_shared_v4(src + x[3]);
-          convert32(c2, sc.y & 0xFFFFu, dst + 32);
-          convert32_bf16(c3, sc.y >> 16, dst + 48);
-          tmem_st_wait();
-          tc_fence_before();
+        // a slot is a stage: the set passes over one slot between its own
+        for (uint32_t i = (odd - st0) & 1u; i < n_st; i += 2) {
+          const uint32_t wc = w0 + i, wi = wc & w_mask;
+          if (!wait_warp(&wfull[wi], (wc >> w_log) & 1u, abort_flag, lim)) { ok = false; break; }
+          if (!stage_free(st0 + i)) { ok = false; break; }
+          if (4 * i + 2 * half < (uint32_t)kb_n) {
+            tc_fence_after();
+            // half a slot: 128 codes and four scales of the row
+            const uint32_t dst = tdst + set * 64;
+            const uint32_t src = sw0 + wi * kCSlot + at * 128 + ((half << 6) ^ x0);
+            const uint2 sc = ld_shared_v2(ss0 + wi * kCScale + at * 16 + half * 8);
+            const uint4 c0 = ld_shared_v4(src + x[0]), c1 = ld_shared_v4(src + x[1]);
+            convert32(c0, sc.x & 0xFFFFu, dst);
+            const uint4 c2 = ld_shared_v4(src + x[2]);
+            convert32(c1, sc.x >> 16, dst + 16);
+            const uint4 c3 = ld_shared_v4(src + x[3]);
+            convert32(c2, sc.y & 0xFFFFu, dst + 32);
+            convert32(c3, sc.y >> 16, dst + 48);
+            tmem_st_wait();
+            tc_fence_before();
+          }
           __syncwarp();
           if (lane == 0) {
             mbar_arrive(&afull[set]);
-            // the warp's rows of the slot are consumed, for two or four sets
-            mbar_arrive_n(&wempty[wi], ((i & 1u) || i + 1 < n_st) ? 2 : 4);
+            mbar_arrive_n(&wempty[wi], 2);  // the warp's rows of the slot are consumed, for two sets
           }
         }
       } else {
         // 64 bf16 weights of each row a slot: every warp passes every slot
         for (uint32_t kb = 0; kb < (uint32_t)kb_n; ++kb) {
-          const uint32_t st = st0 + (kb >> 1);
+          const uint32_t st = st0 + (kb >> 2);
           const uint32_t wc = w0 + kb, wi = wc & w_mask;
-          if (!cwait_warp<20>(&wfull[wi], (wc >> w_log) & 1u, abort_flag, lim)) { ok = false; break; }
-          if ((st & 3u) == (uint32_t)set) {
-            if ((kb & 1u) == 0 && st >= kCOperand &&
-                !cwait_warp<20>(&sempty[(st - kCOperand) & s_mask], ((st - kCOperand) >> s_log) & 1u, abort_flag, lim)) {
-              ok = false;
-              break;
-            }
+          if (!wait_warp(&wfull[wi], (wc >> w_log) & 1u, abort_flag, lim)) { ok = false; break; }
+          if ((st & 1u) == odd && ((kb >> 1) & 1u) == half) {
+            if ((kb & 1u) == 0 && !stage_free(st)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
@@ -794,7 +796,7 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
               const uint4 b2 = ld_shared_v4(src + x[2]), b3 = ld_shared_v4(src + x[3]);
               const uint32_t o[16] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w,
                                       b2.x, b2.y, b2.z, b2.w, b3.x, b3.y, b3.z, b3.w};
-              tmem_st16(tdst + set * (STEPS * 32) + (kb & 1u) * 32 + 16 * p, o);
+              tmem_st16(tdst + set * 64 + (kb & 1u) * 32 + 16 * p, o);
             }
             tmem_st_wait();
             tc_fence_before();
@@ -803,9 +805,14 @@ __global__ void __launch_bounds__(CCfg<Q4>::kThreads, 1)
           }
           if (lane == 0) mbar_arrive(&wempty[wi]);
         }
+        if (!ok) break;
+        if ((kb_n & 3) != 0 && half == 1 && ((st0 + n_st - 1) & 1u) == odd) {  // the last stage's missing half
+          if (!stage_free(st0 + n_st - 1)) break;
+          if (lane == 0) mbar_arrive(&afull[set]);
+        }
       }
       st0 += n_st;
-      w0 += codes ? (n_st + 1) / 2 : kb_n;
+      w0 += codes ? n_st : kb_n;
     }
   }
 
@@ -824,23 +831,23 @@ namespace {
 constexpr int kColsFixed = 1024 + (4 * kCRingMax + 4 + 4 + 2) * 8 + 8 + (4 * kCTable + 1 + 96) * 4;
 constexpr int kColsSmem = 227 * 1024;
 
-template <bool Q4>
+template <bool Q4, int STEPS>
 cudaError_t launch_cols(const CUtensorMap& tmW13, const CUtensorMap& tmW2, const CUtensorMap& tmS13,
                         const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid, cudaStream_t s) {
   static std::atomic<unsigned long long> attr_done{0};
-  cudaError_t e = smem_attr_once(fused_cols_kernel<Q4>, kColsSmem, attr_done);
+  cudaError_t e = smem_attr_once(fused_cols_kernel<Q4, STEPS>, kColsSmem, attr_done);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;  // every CTA resident: see above
   attr[0].val.cooperative = 1;
   cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(CCfg<Q4>::kThreads, 1, 1);
+  cfg.blockDim = dim3(CCfg<Q4, STEPS>::kThreads, 1, 1);
   cfg.dynamicSmemBytes = kColsFixed + a.ring_s * STEPS * ((Q4 ? 0 : kCSlot) + a.b_rows * 128) + a.ring_w * (kCSlot + kCScale);
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fused_cols_kernel<Q4>, tmW13, tmW2, tmS13, tmS2, a, w);
+  return cudaLaunchKernelEx(&cfg, fused_cols_kernel<Q4, STEPS>, tmW13, tmW2, tmS13, tmS2, a, w);
 }
 
 }  // namespace
@@ -858,10 +865,13 @@ void cols_rings(FusedArgs& a, bool q4, int T) {
   a.b_rows = T >= a.tile_tok ? a.tile_tok : (T + 15) / 16 * 16;
   const int room = kColsSmem - kColsFixed;
   if (q4) {
-    a.ring_s = a.b_rows > 32 ? 4 : 8;
-    a.ring_w = room - a.ring_s * STEPS * a.b_rows * 128 >= 8 * (kCSlot + kCScale) ? 8 : 4;
+    a.steps = 4;
+    const int tok = a.steps * a.b_rows * 128;
+    a.ring_s = a.b_rows > 32 ? 2 : 4;
+    a.ring_w = room - a.ring_s * tok >= 8 * (kCSlot + kCScale) ? 8 : 4;
   } else {
-    const int fit = room / (STEPS * (kCSlot + a.b_rows * 128));
+    a.steps = a.b_rows > 16 ? 2 : 4;
+    const int fit = room / (a.steps * (kCSlot + a.b_rows * 128));
     a.ring_s = fit < kCRingMax ? fit : kCRingMax;
     a.ring_w = 0;
   }
@@ -871,8 +881,9 @@ cudaError_t launch_fused_cols(bool q4, const CUtensorMap& tmW13, const CUtensorM
                               const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid,
                               cudaStream_t s) {
   if (grid < 1) return cudaSuccess;
-  return q4 ? launch_cols<true>(tmW13, tmW2, tmS13, tmS2, a, w, grid, s)
-            : launch_cols<false>(tmW13, tmW2, tmS13, tmS2, a, w, grid, s);
+  if (q4) return launch_cols<true, 4>(tmW13, tmW2, tmS13, tmS2, a, w, grid, s);
+  return a.steps == 4 ? launch_cols<false, 4>(tmW13, tmW2, tmS13, tmS2, a, w, grid, s)
+                      : launch_cols<false, 2>(tmW13, tmW2, tmS13, tmS2, a, w, grid, s);
 }
 
 }  // namespace msi

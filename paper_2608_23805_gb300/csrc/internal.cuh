@@ -164,6 +164,7 @@ struct FusedArgs {
   __nv_bfloat16* hs;              // [T, I]
   __nv_bfloat16* ys;              // [T, H]
   int tile_tok;                   // tokens per tile (32, 64 or 128)
+  int steps;                      // 64-K steps per stage (2 or 4)
   int b_rows;                     // token rows per step in a stage (16 .. 128)
   int ring_s, ring_w;             // stages; 4-bit: code slots (both powers of two)
 };

@@ -738,7 +738,7 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 // Weights as MMA rows (gemm_cols.cu), in one launch with a resident call's
 // shared expert, while the groups average fewer rows than a tile holds:
 //   4-bit (one conversion per weight and tile): at 8, 250 and 4,096 tokens of
-//     the Qwen-shaped layer 70, 328 and 520 us against 91, 534 and 546 in two
+//     the Qwen-shaped layer 70, 308 and 520 us against 91, 534 and 546 in two
 //     row-major launches; more than 128 rows take two tiles, two conversions;
 //   bf16: where the launches' latency is what counts (one token: 24 us for
 //     what took 28 + 25 on a side stream); from some 40 tokens on both
