@@ -33,8 +33,8 @@
 // What bounds it: for 4-bit the instructions of the converting and the issuing
 // warps (an MMA of up to 96 columns takes 48 cycles), not HBM; for bf16 and few
 // tokens the latency of a tile's pass over K.  Resident Qwen-shaped layer, both
-// projections: 4-bit 250 tokens 308 us (534 as two row-major launches), 8
-// tokens 70 us (91), 4,096 tokens 520 us (546); bf16 one token 24 us with the
+// projections: 4-bit 250 tokens 300 us (534 as two row-major launches), 8
+// tokens 65 us (91), 4,096 tokens 432 us (546); bf16 one token 24 us with the
 // shared expert (28 without it, which took 25 beside it).
 //
 // Schedule: every CTA takes a contiguous range of the up tiles, then of the
@@ -182,6 +182,11 @@ __device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
 
+__device__ __forceinline__ void st_shared_u16(uint32_t addr, uint32_t v) {
+  asm volatile("{\n\t.reg .b16 h;\n\tcvt.u16.u32 h, %1;\n\tst.shared.b16 [%0], h;\n\t}" ::"r"(addr), "r"(v)
+               : "memory");
+}
+
 __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -297,7 +302,8 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
   uint8_t* sT = smem;
   uint8_t* sW = sT + a.ring_s * stage;   // 4-bit: [ring_w][128][128] codes
   uint8_t* sS = sW + a.ring_w * kCSlot;  // 4-bit: [ring_w][128][8] fp16 scales
-  uint64_t* sfull = reinterpret_cast<uint64_t*>(sS + a.ring_w * kCScale);  // [ring_s]
+  uint8_t* s_epi = sS + a.ring_w * kCScale;  // epilogue staging, 1 KB per warp
+  uint64_t* sfull = reinterpret_cast<uint64_t*>(s_epi + 4096);  // [ring_s]
   uint64_t* sempty = sfull + kCRingMax;
   uint64_t* wfull = sempty + kCRingMax;   // 4-bit: [ring_w]
   uint64_t* wempty = wfull + kCRingMax;
@@ -562,6 +568,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
   } else if (warp < 4) {
     // ------------------------------------------------------------- epilogue
     uint32_t jt = 0;
+    const uint32_t stg = smem_u32(s_epi) + warp * 1024;
     if (a.stall && threadIdx.x == 0) mbar_wait(never, 0, abort_flag, lim);  // runs out: abort
     __syncwarp();
     while (walk.next()) {
@@ -574,9 +581,14 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
       tc_fence_after();
       const uint32_t tb = tmem_base + ((uint32_t)(warp * 32) << 16) + acc * 128;
       const size_t orow = (size_t)(sh ? row0 : s_rb[t.g] + row0);
+      // sixteen tokens at a time through the warp's staging buffer, [token][its
+      // weight rows' bf16], so that a store fills 32 or 64 contiguous bytes a
+      // token with one 16-byte store a lane (a 2- or 4-byte store per token and
+      // lane took the epilogue warps 92 % of the time at 4,096 tokens)
       if (t.up) {
         const int half = lane >> 4;  // 0: the lane's row is a gate row, 1: an up row
-        __nv_bfloat16* out = (sh ? a.hs : a.h) + orow * a.h_ld + t.n * 64 + warp * 16 + (lane & 15);
+        const uint32_t put = stg + half * 32 + (lane & 15) * 2;
+        __nv_bfloat16* out = (sh ? a.hs : a.h) + orow * a.h_ld + t.n * 64 + warp * 16 + (lane & 1) * 8;
 #pragma unroll 1
         for (int c = 0; c < rows; c += 16) {
           uint32_t v[16];
@@ -588,9 +600,13 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
             const uint32_t o = __shfl_xor_sync(0xffffffffu, half ? v[2 * i] : v[2 * i + 1], 16);
             const float g = __uint_as_float(half ? o : v[2 * i]);
             const float u = __uint_as_float(half ? v[2 * i + 1] : o);
-            const int tok = c + 2 * i + half;
-            if (tok < rows) out[(size_t)tok * a.h_ld] = __float2bfloat16_rn(silu_mul(g, u));
+            st_shared_u16(put + i * 64, pack_bf16x2(silu_mul(g, u), 0.f));
           }
+          __syncwarp();
+          const int tok = c + (lane >> 1);
+          const uint4 q = ld_shared_v4(stg + lane * 16);
+          if (tok < rows) *reinterpret_cast<uint4*>(out + (size_t)tok * a.h_ld) = q;
+          __syncwarp();
         }
         // publish the warp's part of the tile: its h stores, then one release
         // add on the token tile's counter
@@ -598,8 +614,8 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
         __syncwarp();
         if (lane == 0) red_release_gpu_add(&a.ready[s_mt[t.g] + t.m], 1);
       } else {
-        const int odd = lane & 1;
-        __nv_bfloat16* out = (sh ? a.ys : a.y) + orow * a.y_ld + t.n * 128 + warp * 32 + (lane & ~1);
+        const uint32_t put = stg + lane * 2;
+        __nv_bfloat16* out = (sh ? a.ys : a.y) + orow * a.y_ld + t.n * 128 + warp * 32 + (lane & 3) * 8;
 #pragma unroll 1
         for (int c = 0; c < rows; c += 16) {
           uint32_t v[16];
@@ -607,13 +623,18 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
           tmem_ld_wait(v);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            // even lanes store the even token's two features, odd lanes the odd's
-            const uint32_t o = __shfl_xor_sync(0xffffffffu, odd ? v[2 * i] : v[2 * i + 1], 1);
-            const float lo = __uint_as_float(odd ? o : v[2 * i]);
-            const float hi = __uint_as_float(odd ? v[2 * i + 1] : o);
-            const int tok = c + 2 * i + odd;
-            if (tok < rows) *reinterpret_cast<uint32_t*>(out + (size_t)tok * a.y_ld) = pack_bf16x2(lo, hi);
+            const uint32_t p = pack_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+            st_shared_u16(put + i * 128, p);
+            st_shared_u16(put + i * 128 + 64, p >> 16);
           }
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int tok = c + 8 * j + (lane >> 2);
+            const uint4 q = ld_shared_v4(stg + j * 512 + lane * 16);
+            if (tok < rows) *reinterpret_cast<uint4*>(out + (size_t)tok * a.y_ld) = q;
+          }
+          __syncwarp();
         }
       }
       tc_fence_before();
@@ -828,7 +849,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
 
 namespace {
 
-constexpr int kColsFixed = 1024 + (4 * kCRingMax + 4 + 4 + 2) * 8 + 8 + (4 * kCTable + 1 + 96) * 4;
+constexpr int kColsFixed = 1024 + 4096 + (4 * kCRingMax + 4 + 4 + 2) * 8 + 8 + (4 * kCTable + 1 + 96) * 4;
 constexpr int kColsSmem = 227 * 1024;
 
 template <bool Q4, int STEPS>

@@ -736,18 +736,22 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 }
 
 // Weights as MMA rows (gemm_cols.cu), in one launch with a resident call's
-// shared expert, while the groups average fewer rows than a tile holds:
-//   4-bit (one conversion per weight and tile): at 8, 250 and 4,096 tokens of
-//     the Qwen-shaped layer 70, 308 and 520 us against 91, 534 and 546 in two
-//     row-major launches; more than 128 rows take two tiles, two conversions;
+// shared expert, while the groups average few rows:
+//   4-bit: at 8, 250 and 4,096 tokens of the Qwen-shaped layer 65, 300 and 432
+//     us against 91, 534 and 546 in two row-major launches; the call at 8,192
+//     tokens 990 against 1,209, at 20,000 (390 rows a group, four tiles and
+//     conversions) 2,105 against 2,215, at 32,768 3,508 against 3,086 on pairs.
+//     A wave up to 256 rows.
 //   bf16: where the launches' latency is what counts (one token: 24 us for
-//     what took 28 + 25 on a side stream); from some 40 tokens on both
+//     what took 28 + 25 on a side stream).  From some 40 tokens on both
 //     orientations stream the weights at the same rate (0.97 of HBM), and the
-//     row-major tiles read the tokens half as often.  Not a wave: its launch
-//     has no shared expert to take in.
-constexpr long long kColsMaxRows = 128, kColsMaxRowsBf16 = 8;
+//     row-major tiles read the tokens half as often (the call at 250 tokens 524
+//     in both, at 600 545 row-major, 555 here).  Not a wave: its launch has no
+//     shared expert to take in.
+constexpr long long kColsMaxRows = 512, kColsMaxRowsWave = 256, kColsMaxRowsBf16 = 8;
 bool cols_tiles(const msi_plan* p, const FwdCtx& f, long long rows, int ng, bool wave = false) {
-  return !(f.flags & (MSI_FWD_SPLIT_WAVES | MSI_FWD_SINGLE_CTA)) && ng > 0 && rows < kColsMaxRows * ng &&
+  return !(f.flags & (MSI_FWD_SPLIT_WAVES | MSI_FWD_SINGLE_CTA)) && ng > 0 &&
+         rows < (wave ? kColsMaxRowsWave : kColsMaxRows) * ng &&
          (p->d.wdtype == MSI_W_Q4G32 || (!wave && rows < kColsMaxRowsBf16 * ng));
 }
 
