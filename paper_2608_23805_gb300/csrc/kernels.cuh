@@ -153,7 +153,10 @@ struct CombineArgs {
 // ---------------------------------------------------------------------------
 // Launchers (asynchronous on the given stream; return the launch error)
 // ---------------------------------------------------------------------------
-cudaError_t launch_router(const RouterArgs& a, cudaStream_t s);
+// The FFMA router; sa (only where router_scatters): it scatters as well, with
+// the resident call's table from tp.
+bool router_scatters(int E, int T);
+cudaError_t launch_router(const RouterArgs& a, const ScatterArgs* sa, const TableParams& tp, cudaStream_t s);
 cudaError_t launch_router_logits(const CUtensorMap& tmX, const RouterTcArgs& a, const TableParams& tp,
                                  cudaStream_t s);
 // sa not null: a call of at most kFuseTokens tokens is scattered as well (no

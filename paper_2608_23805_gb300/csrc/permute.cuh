@@ -85,4 +85,50 @@ __device__ __forceinline__ void build_groups(const ScatterArgs& a, int e, int cn
   }
 }
 
+// The scatter's work for a whole call of at most kFuseTokens tokens, by one
+// block of at least kMaxExperts threads once every id is written: offsets,
+// counts, permutation and, for a resident call, the generation re-check (slot
+// and code of the thread's expert) and the GEMM groups.  A token names an
+// expert at most once, so an expert's rows are the set bits of its token mask:
+// counts and stable ranks are population counts.
+struct ScatterShared {
+  unsigned mask[kFuseTokens / 32][kMaxExperts];
+  int offs[kMaxExperts];
+  int tmp[32];
+};
+__device__ __forceinline__ void scatter_call(const int* ids, int T, int k, int E, const ScatterArgs& s, bool resident,
+                                             int slot, int code, ScatterShared& sh) {
+  const int tid = threadIdx.x, e = tid, nw = (T + 31) / 32;
+  if (tid < kMaxExperts)
+    for (int w = 0; w < nw; ++w) sh.mask[w][tid] = 0u;
+  for (int r = tid; r < s.n_ready; r += blockDim.x) s.ready[r] = 0;
+  __syncthreads();
+  const int n = T * k;
+  for (int f = tid; f < n; f += blockDim.x) {
+    const int tok = f / k;
+    atomicOr(&sh.mask[tok >> 5][__ldcg(&ids[f])], 1u << (tok & 31));
+  }
+  __syncthreads();
+  int cnt = 0;
+  if (e < E)
+    for (int w = 0; w < nw; ++w) cnt += __popc(sh.mask[w][e]);
+  int total;
+  const int base = block_excl_scan(cnt, sh.tmp, &total);
+  if (e < E) {
+    sh.offs[e] = base;
+    s.offsets[e] = base;
+    s.counts_out[e] = cnt;
+  }
+  if (tid == 0) s.offsets[E] = total;
+  __syncthreads();
+  for (int f = tid; f < n; f += blockDim.x) {
+    const int tok = f / k, id = __ldcg(&ids[f]), w = tok >> 5;
+    int pos = sh.offs[id] + __popc(sh.mask[w][id] & ((1u << (tok & 31)) - 1u));  // + the expert's earlier tokens
+    for (int q = 0; q < w; ++q) pos += __popc(sh.mask[q][id]);
+    s.perm[pos] = tok;
+    s.inv[f] = pos;
+  }
+  if (resident) build_groups(s, e, cnt, base, slot, cnt > 0 ? code : 0, sh.tmp);
+}
+
 }  // namespace msi

@@ -855,8 +855,13 @@ msi_status route_rows(msi_plan* p, FwdCtx& f, const float* rw, const msi_route_e
     ra.sh = first && d.has_shared ? at<Group>(ws, L.sh_group) : nullptr;
     ra.sh_total = at<int>(ws, L.sh_total);
     ra.shared_slot = tp.shared_slot;
-    LAUNCH(p, MSI_K_ROUTER, s, launch_router(ra, s));
+    const bool fuse = first && xa != nullptr && router_scatters(E, f.T);
+    LAUNCH(p, MSI_K_ROUTER, s, launch_router(ra, fuse ? xa : nullptr, tp, s));
     if (first && d.has_shared) CK(cudaEventRecord(p->ev_fork, s));  // this router begins the forward itself
+    if (fuse) {
+      *scattered = true;
+      return MSI_OK;
+    }
   }
   // the column scan (per-block prefixes and counts); a small forward's
   // scatter takes it over (scan = false)
@@ -956,7 +961,7 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
   bool scattered = false;
   msi_status st = route_rows(p, f, f.router_w, f.ev, true, tp, f.cs, !fuse_scan, &xa, &scattered);
   if (st != MSI_OK) return st;
-  if (tp.E > 0 && !tensor_router(d))
+  if (tp.E > 0 && !tensor_router(d) && !scattered)
     LAUNCH(p, MSI_K_UPLOAD, f.cs, launch_upload(tp, at<int>(ws, L.table), at<unsigned long long>(ws, L.expected),
                             nullptr, nullptr, nullptr, f.cs));
   if (!scattered) LAUNCH(p, MSI_K_SCATTER, f.cs, launch_scatter(xa, f.cs));

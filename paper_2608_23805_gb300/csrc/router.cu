@@ -17,7 +17,7 @@
 // one k-quad hit all 32 banks once per 8 lanes.  Accumulation runs over h in
 // ascending order.  Top-k: one warp per token, k+1 rounds of a warp-shuffle
 // argmax over (logit desc, id asc).
-#include "kernels.cuh"
+#include "permute.cuh"
 
 namespace msi {
 
@@ -63,12 +63,13 @@ __device__ __forceinline__ void load_stage(const RouterArgs& a, uint8_t* st, int
 }
 
 // Top-k, softmax weights, gap and shared gate of the block's tokens from the
-// logits L[TM][lld] in shared memory (each warp TM / warps tokens), then the
-// block's expert histogram.  ids_s: shared scratch [TM * k].  NV: logits per
-// lane (E <= 32 NV).
+// logits L[TM][lld] in shared memory (each warp TM / warps tokens), then, with
+// `count`, the block's expert histogram.  ids_s: shared scratch [TM * k].  NV:
+// logits per lane (E <= 32 NV).  A NaN logit ranks as -inf, so that every id
+// names an expert.
 template <int NV>
 __device__ __forceinline__ void select_and_count(const RouterArgs& a, const float* L, int lld, int* ids_s,
-                                                 int t0) {
+                                                 int t0, bool count = true) {
   const int tid = threadIdx.x;
   // top-k: warp w handles tokens w*tpw .. w*tpw+tpw-1
   const int warp = tid >> 5, lane = tid & 31;
@@ -84,6 +85,7 @@ __device__ __forceinline__ void select_and_count(const RouterArgs& a, const floa
     for (int i = 0; i < NV; ++i) {
       const int e = lane + 32 * i;
       v[i] = (i < per_lane && e < a.E) ? L[tok * lld + e] : -INFINITY;
+      if (v[i] != v[i]) v[i] = -INFINITY;
     }
     uint32_t removed = 0;
     float my_v = -INFINITY;
@@ -147,6 +149,7 @@ __device__ __forceinline__ void select_and_count(const RouterArgs& a, const floa
     }
   }
   __syncthreads();
+  if (!count) return;
 
   // per-block histogram of the routed ids (deterministic, no atomics)
   const int nids = nvalid * k;
@@ -249,7 +252,8 @@ struct SmallCfg {
 };
 
 template <int EL>
-__global__ void __launch_bounds__(SmallCfg<EL>::kThreads, 1) router_small_kernel(const RouterArgs a) {
+__global__ void __launch_bounds__(SmallCfg<EL>::kThreads, 1)
+    router_small_kernel(const RouterArgs a, const ScatterArgs s, const __grid_constant__ TableParams tp) {
   using C = SmallCfg<EL>;
   // the forward's first kernel (status null: a prediction pass)
   if (blockIdx.x == 0 && threadIdx.x == 0 && a.status != nullptr)
@@ -294,7 +298,23 @@ __global__ void __launch_bounds__(SmallCfg<EL>::kThreads, 1) router_small_kernel
   }
   L[tok * kSmallLLD + e] = acc;
   __syncthreads();
-  select_and_count<1>(a, L, kSmallLLD, ids_s, t0);
+  if (s.ids == nullptr) {
+    select_and_count<1>(a, L, kSmallLLD, ids_s, t0);
+    return;
+  }
+  // the whole call in this launch (one cluster of blocks): after every block's
+  // ids are written, the first block does the scatter's work
+  select_and_count<1>(a, L, kSmallLLD, ids_s, t0, false);
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (blockIdx.x != 0) return;
+  __shared__ ScatterShared sh;
+  int slot = -1, code = 0;
+  if (tid < tp.E) {
+    slot = tp.slot[tid];
+    code = check_code(s.genwords, slot, s.layer, tid, tp.expected[tid]);
+  }
+  scatter_call(a.ids, a.T, a.k, a.E, s, tp.E > 0, slot, code, sh);
 }
 
 }  // namespace
@@ -313,7 +333,7 @@ static cudaError_t launch_ep(const RouterArgs& a, cudaStream_t s) {
 }
 
 template <int EL>
-static cudaError_t launch_small(const RouterArgs& a, cudaStream_t s) {
+static cudaError_t launch_small(const RouterArgs& a, const ScatterArgs* sa, const TableParams& tp, cudaStream_t s) {
   using C = SmallCfg<EL>;
   static std::atomic<unsigned long long> attr_done{0};
   {
@@ -322,13 +342,32 @@ static cudaError_t launch_small(const RouterArgs& a, cudaStream_t s) {
   }
   const int nb = (a.T + TM - 1) / TM;
   if (nb == 0) return cudaSuccess;
-  router_small_kernel<EL><<<nb, C::kThreads, C::kSmem, s>>>(a);
-  return cudaGetLastError();
+  static const ScatterArgs none{};
+  if (sa == nullptr) {
+    router_small_kernel<EL><<<nb, C::kThreads, C::kSmem, s>>>(a, none, tp);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = nb;  // kFuseTokens / TM = 8 at most
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(nb, 1, 1);
+  cfg.blockDim = dim3(C::kThreads, 1, 1);
+  cfg.dynamicSmemBytes = C::kSmem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, router_small_kernel<EL>, a, *sa, tp);
 }
 
-cudaError_t launch_router(const RouterArgs& a, cudaStream_t s) {
-  if (a.E <= 16) return launch_small<16>(a, s);
-  if (a.E <= 32) return launch_small<32>(a, s);
+// The small kernel does a short call's scatter too (one launch instead of
+// three for a resident call of 64 tokens: router, table upload, scatter).
+bool router_scatters(int E, int T) { return E <= 32 && T <= kFuseTokens; }
+
+cudaError_t launch_router(const RouterArgs& a, const ScatterArgs* sa, const TableParams& tp, cudaStream_t s) {
+  if (a.E <= 16) return launch_small<16>(a, sa, tp, s);
+  if (a.E <= 32) return launch_small<32>(a, sa, tp, s);
   return a.E <= 64 ? launch_ep<64>(a, s) : launch_ep<512>(a, s);
 }
 

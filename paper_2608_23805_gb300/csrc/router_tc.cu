@@ -518,9 +518,7 @@ template <int NV>
 __global__ void __launch_bounds__(512, 2) router_select_scatter_kernel(const RouterTcArgs a,
                                                                        const ScatterArgs s) {
   constexpr int kTok = 8;
-  __shared__ unsigned mask[kFuseTokens / 32][kMaxExperts];
-  __shared__ int offs[kMaxExperts];
-  __shared__ int tmp[32];
+  __shared__ ScatterShared sh;
   __shared__ int s_last;
   __shared__ SelectScratch scratch[kTok];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -541,36 +539,7 @@ __global__ void __launch_bounds__(512, 2) router_select_scatter_kernel(const Rou
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const int nw = (a.T + 31) / 32;
-  for (int w = 0; w < nw; ++w) mask[w][tid] = 0u;
-  for (int r = tid; r < s.n_ready; r += blockDim.x) s.ready[r] = 0;
-  __syncthreads();
-  const int n = a.T * a.k;
-  for (int f = tid; f < n; f += blockDim.x) {
-    const int tok = f / a.k;
-    atomicOr(&mask[tok >> 5][__ldcg(&a.ids[f])], 1u << (tok & 31));
-  }
-  __syncthreads();
-  int cnt = 0;
-  if (e < a.E)
-    for (int w = 0; w < nw; ++w) cnt += __popc(mask[w][e]);
-  int total;
-  const int base = block_excl_scan(cnt, tmp, &total);
-  offs[e] = base;
-  if (e < a.E) {
-    s.offsets[e] = base;
-    s.counts_out[e] = cnt;
-  }
-  if (tid == 0) s.offsets[a.E] = total;
-  __syncthreads();
-  for (int f = tid; f < n; f += blockDim.x) {
-    const int tok = f / a.k, id = __ldcg(&a.ids[f]), w = tok >> 5;
-    int pos = offs[id] + __popc(mask[w][id] & ((1u << (tok & 31)) - 1u));  // + the expert's earlier tokens
-    for (int q = 0; q < w; ++q) pos += __popc(mask[q][id]);
-    s.perm[pos] = tok;
-    s.inv[f] = pos;
-  }
-  if (s.tab_slot != nullptr) build_groups(s, e, cnt, base, slot, cnt > 0 ? code : 0, tmp);
+  scatter_call(a.ids, a.T, a.k, a.E, s, s.tab_slot != nullptr, slot, code, sh);
 }
 
 template <int CH, bool STACK>

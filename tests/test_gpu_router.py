@@ -63,7 +63,8 @@ def inputs(T, E, H, seed=0):
     g = torch.Generator(device="cuda").manual_seed(seed)
     x = torch.randn(T, H, generator=g, device="cuda").to(torch.bfloat16)
     wr = torch.randn(E, H, generator=g, device="cuda") * 0.02
-    wr[E // 2:E // 2 + 4] = wr[:4]  # exact ties between experts
+    n = min(4, E // 2)
+    wr[E // 2:E // 2 + n] = wr[:n]  # exact ties between experts
     x[T // 2] = 0                   # and over all of them
     return x, wr
 
@@ -104,3 +105,24 @@ def test_misaligned_router_weights(T):
     off.copy_(wr)
     assert off.data_ptr() % 16 == 4
     check(x, off, 10, route(x, off, 512, 10, 512))
+
+
+@pytest.mark.parametrize("E,k,H", [(16, 2, 256), (5, 5, 512), (20, 3, 256), (32, 10, 1024)])
+@pytest.mark.parametrize("T", [1, 32, 33, 200, 256, 257])
+def test_small_layers(T, E, k, H):
+    # up to 256 rows the selecting launch scatters too (a cluster of 32-row blocks)
+    x, wr = inputs(T, E, H, 4)
+    check(x, wr, k, route(x, wr, E, k, H, shared=T == 33))
+
+
+@pytest.mark.parametrize("E,H", [(16, 256), (512, 512)])
+@pytest.mark.parametrize("T", [40, 700])
+def test_nan_rows_name_experts(T, E, H):
+    # a row without an order still names k different experts, and the others
+    # are not touched
+    x, wr = inputs(T, E, H, 5)
+    x[3] = float("nan")
+    ids, w, counts, _ = route(x, wr, E, 2, H)
+    assert ids.min() >= 0 and ids.max() < E and (ids[:, 0] != ids[:, 1]).all()
+    assert (counts == np.bincount(ids.ravel(), minlength=E)).all()
+    assert np.isfinite(np.delete(w, 3, 0)).all()
