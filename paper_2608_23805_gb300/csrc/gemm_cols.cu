@@ -354,6 +354,8 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
       tma_prefetch(&tmS2);
     }
   }
+  grid_wait();
+  grid_release();
   // the previous wave's counters, zeroed for the next wave
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.n_ready_clear; r += gridDim.x * blockDim.x)
     a.ready_clear[r] = 0;
@@ -854,20 +856,23 @@ constexpr int kColsSmem = 227 * 1024;
 
 template <bool Q4, int STEPS>
 cudaError_t launch_cols(const CUtensorMap& tmW13, const CUtensorMap& tmW2, const CUtensorMap& tmS13,
-                        const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid, cudaStream_t s) {
+                        const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid, bool after,
+                        cudaStream_t s) {
   static std::atomic<unsigned long long> attr_done{0};
   cudaError_t e = smem_attr_once(fused_cols_kernel<Q4, STEPS>, kColsSmem, attr_done);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeCooperative;  // every CTA resident: see above
   attr[0].val.cooperative = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(CCfg<Q4, STEPS>::kThreads, 1, 1);
   cfg.dynamicSmemBytes = kColsFixed + a.ring_s * STEPS * ((Q4 ? 0 : kCSlot) + a.b_rows * 128) + a.ring_w * (kCSlot + kCScale);
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = after ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, fused_cols_kernel<Q4, STEPS>, tmW13, tmW2, tmS13, tmS2, a, w);
 }
 
@@ -900,11 +905,11 @@ void cols_rings(FusedArgs& a, bool q4, int T) {
 
 cudaError_t launch_fused_cols(bool q4, const CUtensorMap& tmW13, const CUtensorMap& tmW2, const CUtensorMap& tmS13,
                               const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid,
-                              cudaStream_t s) {
+                              bool after, cudaStream_t s) {
   if (grid < 1) return cudaSuccess;
-  if (q4) return launch_cols<true, 4>(tmW13, tmW2, tmS13, tmS2, a, w, grid, s);
-  return a.steps == 4 ? launch_cols<false, 4>(tmW13, tmW2, tmS13, tmS2, a, w, grid, s)
-                      : launch_cols<false, 2>(tmW13, tmW2, tmS13, tmS2, a, w, grid, s);
+  if (q4) return launch_cols<true, 4>(tmW13, tmW2, tmS13, tmS2, a, w, grid, after, s);
+  return a.steps == 4 ? launch_cols<false, 4>(tmW13, tmW2, tmS13, tmS2, a, w, grid, after, s)
+                      : launch_cols<false, 2>(tmW13, tmW2, tmS13, tmS2, a, w, grid, after, s);
 }
 
 }  // namespace msi

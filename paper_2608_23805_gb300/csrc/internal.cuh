@@ -30,6 +30,26 @@ inline cudaError_t smem_attr_once(K* kernel, int bytes, std::atomic<unsigned lon
   return e;
 }
 
+// A launch that may overlap the end of its predecessor in the stream (see
+// grid_wait), where that is a kernel and nothing stands between them but event
+// records: an event wait there has to hold for the whole launch.  after =
+// false: an ordinary launch.
+template <typename... P, typename... A>
+inline cudaError_t launch_after(bool after, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = after ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---------------------------------------------------------------------------
 // Limits of the kernels
 // ---------------------------------------------------------------------------
@@ -198,7 +218,7 @@ int cols_tile_tokens(long long rows, int groups);
 void cols_rings(FusedArgs& a, bool q4, int T);
 cudaError_t launch_fused_cols(bool q4, const CUtensorMap& tmW13, const CUtensorMap& tmW2, const CUtensorMap& tmS13,
                               const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid,
-                              cudaStream_t s);
+                              bool after, cudaStream_t s);
 
 // GEMM tiling
 constexpr int kBM = 128;
@@ -534,6 +554,14 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
       "h"(mask)
       : "memory");
 }
+
+// Programmatic dependent launch: a kernel launched with launch_after may start
+// while its predecessor in the stream still runs, and must not touch global
+// memory before grid_wait, which returns when the predecessor has completed and
+// its writes are visible.  Every kernel of such a chain waits, so each follows
+// all before it.  grid_release lets the successor start.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // One lane of a converged warp, the same one each time.  The MMA warps run
 // their loops with all lanes and issue under this predicate: in a branch on

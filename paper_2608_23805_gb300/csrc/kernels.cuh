@@ -185,7 +185,8 @@ struct StageCopyArgs {
   int parts;                     // blocks per extent
 };
 cudaError_t launch_stage_copy(const StageCopyArgs& a, GenWord* genwords, cudaStream_t s);
-cudaError_t launch_combine(const CombineArgs& a, cudaStream_t s);
+// after: the predecessor in the stream is a kernel (launch_after).
+cudaError_t launch_combine(const CombineArgs& a, bool after, cudaStream_t s);
 cudaError_t launch_zero_counts(int* counts, int E, cudaStream_t s);
 
 #ifdef __CUDACC__

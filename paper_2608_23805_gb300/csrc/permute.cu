@@ -20,6 +20,8 @@ namespace {
 // ---- column prefix over router blocks: bbase[b][e], counts[e] ----
 __global__ void __launch_bounds__(1024) colscan_kernel(const ScanArgs a) {
   __shared__ int part[32][33];
+  grid_wait();
+  grid_release();
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int e = blockIdx.x * 32 + tx;
   const int sz = (a.nb + 31) / 32;
@@ -139,6 +141,8 @@ __global__ void __launch_bounds__(kScatterWarps * 32) scatter_kernel(const Scatt
   __shared__ int run[kScatterWarps][kMaxExperts];
   __shared__ int wsum[kScatterWarps];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  grid_wait();
+  grid_release();
 
   // exclusive scan of counts (E <= 512, 128 threads x 4 values); with
   // fuse_scan the counts are the column sums of the router blocks' counts
@@ -361,10 +365,13 @@ __device__ __forceinline__ void fma8(float (&acc)[8], float w, const uint4& y) {
 // summed (still in j order, fp32), so each thread keeps eight 16-byte loads
 // in flight.
 __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs a) {
-  if (*a.status != 0) return;  // fail closed: nothing stale becomes visible
+  grid_wait();
   __shared__ int s_row[kMaxTopK];
   __shared__ float s_w[kMaxTopK];
   const int t = blockIdx.x;
+  // fail closed: nothing stale becomes visible.  Checked before the stores: the
+  // rows' indices are a bijection in any case, and the load need not come first
+  const int status = *a.status;
   if (threadIdx.x < a.k) {
     s_row[threadIdx.x] = __ldg(&a.inv[(size_t)t * a.k + threadIdx.x]);
     s_w[threadIdx.x] = __ldg(&a.weights[(size_t)t * a.k + threadIdx.x]);
@@ -409,6 +416,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs a) {
       acc[6] += bf16_lo(y.w);
       acc[7] += bf16_hi(y.w);
     }
+    if (status != 0) return;
     uint4 o;
     o.x = pack_bf16x2(acc[0], acc[1]);
     o.y = pack_bf16x2(acc[2], acc[3]);
@@ -425,14 +433,12 @@ __global__ void zero_kernel(int* p, int n) {
 }  // namespace
 
 cudaError_t launch_colscan(const ScanArgs& a, cudaStream_t s) {
-  colscan_kernel<<<(a.E + 31) / 32, dim3(32, 32), 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_after(true, colscan_kernel, (a.E + 31) / 32, dim3(32, 32), 0, s, a);
 }
 
 cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s) {
   const int grid = (a.nb + kScatterWarps - 1) / kScatterWarps + 1;  // + the setup block
-  scatter_kernel<<<grid, kScatterWarps * 32, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_after(true, scatter_kernel, grid, kScatterWarps * 32, 0, s, a);
 }
 
 cudaError_t launch_upload(const TableParams& p, int* table, unsigned long long* expected, int* status,
@@ -459,11 +465,10 @@ cudaError_t launch_stage_copy(const StageCopyArgs& a, GenWord* genwords, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_combine(const CombineArgs& a, cudaStream_t s) {
+cudaError_t launch_combine(const CombineArgs& a, bool after, cudaStream_t s) {
   if (a.T == 0) return cudaSuccess;
   const int nthreads = min(256, a.H / 8);
-  combine_kernel<<<a.T, nthreads, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_after(after, combine_kernel, a.T, nthreads, 0, s, a);
 }
 
 cudaError_t launch_zero_counts(int* counts, int E, cudaStream_t s) {

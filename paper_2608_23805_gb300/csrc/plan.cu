@@ -1128,7 +1128,7 @@ msi_status routed_ffn(msi_plan* p, FwdCtx& f, int ng, int grid1, int grid2, long
       const int grid = (int)std::min<long long>(p->sms - spare, std::max<long long>(1, all));
       LAUNCH(p, MSI_K_FFN, f.cs,
              launch_fused_cols(!bf16, p->tm_p13, bf16 ? p->tm_w2 : p->tm_c2, d.has_shared ? p->tm_psh13 : p->tm_p13,
-                               d.has_shared ? p->tm_sh2 : p->tm_p13, fa, wv, grid, f.cs));
+                               d.has_shared ? p->tm_sh2 : p->tm_p13, fa, wv, grid, wp == nullptr, f.cs));
       return MSI_OK;
     }
     if (!bf16) {
@@ -1205,7 +1205,8 @@ msi_status shared_ffn(msi_plan* p, FwdCtx& f, cudaStream_t stream) {
   return MSI_OK;
 }
 
-msi_status finish(msi_plan* p, FwdCtx& f) {
+// after: nothing but event records since the compute stream's last kernel
+msi_status finish(msi_plan* p, FwdCtx& f, bool after) {
   const auto& d = p->d;
   if (f.T > 0) {
     // host-buffer calls combine in row chunks; each chunk's rows go back
@@ -1228,7 +1229,7 @@ msi_status finish(msi_plan* p, FwdCtx& f) {
       c.H = H;
       c.k = k;
       c.status = at<int>(f.ws, f.L.status);
-      LAUNCH(p, MSI_K_COMBINE, f.cs, launch_combine(c, f.cs));
+      LAUNCH(p, MSI_K_COMBINE, f.cs, launch_combine(c, after, f.cs));
       if (f.out_host != nullptr) {
         CK(cudaEventRecord(p->ev_io_a, f.cs));
         CK(cudaStreamWaitEvent(f.io, p->ev_io_a, 0));
@@ -1586,7 +1587,7 @@ msi_status forward_resident(msi_plan* p, int layer, const void* x, int T, const 
     if (st != MSI_OK) return st;
   }
   if (fork) CK(cudaStreamWaitEvent(f.cs, p->ev_join, 0));
-  st = finish(p, f);
+  st = finish(p, f, !fork);
   if (st != MSI_OK) return st;
   p->ctr.forwards++;
   return MSI_OK;
@@ -1981,7 +1982,7 @@ msi_status forward_streamed(msi_plan* p, int layer, const void* x, int T, const 
     CK(cudaStreamWaitEvent(f.cs, p->ev_pjoin, 0));
     pred_join.ev = nullptr;
   }
-  st = finish(p, f);
+  st = finish(p, f, !predict);
   if (st != MSI_OK) return st;
   p->ctr.forwards++;
   p->ctr.streamed_forwards++;

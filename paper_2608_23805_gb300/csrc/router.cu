@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(SmallCfg<EL>::kThreads, 1)
   // the forward's first kernel (status null: a prediction pass)
   if (blockIdx.x == 0 && threadIdx.x == 0 && a.status != nullptr)
     forward_begin(a.status, a.sh, a.sh_total, a.T, a.shared_slot);
+  grid_release();
   extern __shared__ __align__(128) uint8_t smem[];
   float4* wt = reinterpret_cast<float4*>(smem);
   __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(smem + C::kWT);

@@ -182,6 +182,7 @@ __global__ void __launch_bounds__(kRlThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
+  grid_release();
   if (warp == kCvtWarps) {
     // ------------------------------------------------------------- x tiles (TMA)
     if (lane == 0) {
@@ -494,6 +495,8 @@ __global__ void __launch_bounds__(512, 2) router_select_kernel(const RouterTcArg
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int e = threadIdx.x; e < a.E; e += blockDim.x) hist[e] = 0;
   __syncthreads();
+  grid_wait();
+  grid_release();
 #pragma unroll 1
   for (int u = 0; u < 2; ++u) {
     const int t = a.t0 + blockIdx.x * 32 + u * 16 + warp;
@@ -523,6 +526,8 @@ __global__ void __launch_bounds__(512, 2) router_select_scatter_kernel(const Rou
   __shared__ SelectScratch scratch[kTok];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int e = tid;
+  grid_wait();
+  grid_release();
   int slot = -1, code = 0;
   if (s.tab_slot != nullptr && e < a.E) {
     slot = s.tab_slot[e];
@@ -533,12 +538,16 @@ __global__ void __launch_bounds__(512, 2) router_select_scatter_kernel(const Rou
     if (warp < kTok) select_token<NV>(a, t, lane, scratch[warp]);
     else if (a.wsg != nullptr) shared_gate(a, t, lane);
   }
-  __threadfence();  // the ids, before the ticket
-  __syncthreads();
-  if (tid == 0) s_last = atomicAdd(s.ticket, 1) == (int)gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
+  if (gridDim.x > 1) {
+    __threadfence();  // the ids, before the ticket
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(s.ticket, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+  } else {
+    __syncthreads();
+  }
   scatter_call(a.ids, a.T, a.k, a.E, s, s.tab_slot != nullptr, slot, code, sh);
 }
 
@@ -554,9 +563,9 @@ cudaError_t launch_logits(const CUtensorMap& tmX, const RouterTcArgs& a, const T
 }
 
 template <int NV>
-void select_nv(const RouterTcArgs& a, const ScatterArgs* sa, cudaStream_t s) {
-  if (sa != nullptr) router_select_scatter_kernel<NV><<<(a.T + 7) / 8, 512, 0, s>>>(a, *sa);
-  else router_select_kernel<NV><<<(a.rows + 31) / 32, 512, 0, s>>>(a);
+cudaError_t select_nv(const RouterTcArgs& a, const ScatterArgs* sa, cudaStream_t s) {
+  if (sa != nullptr) return launch_after(true, router_select_scatter_kernel<NV>, (a.T + 7) / 8, 512, 0, s, a, *sa);
+  return launch_after(true, router_select_kernel<NV>, (a.rows + 31) / 32, 512, 0, s, a);
 }
 
 }  // namespace
@@ -600,10 +609,9 @@ cudaError_t launch_router_logits(const CUtensorMap& tmX, const RouterTcArgs& a, 
 
 cudaError_t launch_router_select(const RouterTcArgs& a, const ScatterArgs* sa, cudaStream_t s) {
   const int nv = (a.E + 127) / 128;
-  if (nv <= 1) select_nv<1>(a, sa, s);
-  else if (nv <= 2) select_nv<2>(a, sa, s);
-  else select_nv<4>(a, sa, s);
-  return cudaGetLastError();
+  if (nv <= 1) return select_nv<1>(a, sa, s);
+  if (nv <= 2) return select_nv<2>(a, sa, s);
+  return select_nv<4>(a, sa, s);
 }
 
 }  // namespace msi
