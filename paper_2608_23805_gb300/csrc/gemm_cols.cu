@@ -27,14 +27,21 @@
 //       The weights thus cross shared memory once, as codes: converted in
 //       shared memory they would cost 4 x their bf16 size in shared-memory
 //       traffic, which bounds the row-major 4-bit kernel.
-// Tokens (operand B): cp.async of the tile's rows only (x through the
-// permutation, or h) into the stage, in the 128-byte swizzle.
+// Tokens (operand B), in the 128-byte swizzle, the tile's rows only: h by TMA in
+// boxes of 16 rows; x through the permutation, by TMA gathers of four rows up to
+// 64 tokens a tile, else by cp.async.  Copies and gathers by size (a call, us):
+//   tokens               37    250    800   1,600   4,096
+//   cp.async, x and h   195    346    382     421     537
+//   gathers for x       187    334    369     427     562
+//   cp.async for x      -       352    382     406     521
+// A gather frees the schedulers that the conversion needs, but brings fewer
+// bytes a cycle than 128 threads' copies, which is what counts in large tiles.
 //
 // What bounds it: for 4-bit the instructions of the converting and the issuing
 // warps (an MMA of up to 96 columns takes 48 cycles), not HBM; for bf16 and few
 // tokens the latency of a tile's pass over K.  Resident Qwen-shaped layer, both
-// projections: 4-bit 250 tokens 300 us (534 as two row-major launches), 8
-// tokens 65 us (91), 4,096 tokens 432 us (546); bf16 one token 24 us with the
+// projections: 4-bit 250 tokens 288 us (534 as two row-major launches), 8
+// tokens 62 us (91), 4,096 tokens 416 us (546); bf16 one token 24 us with the
 // shared expert (28 without it, which took 25 beside it).
 //
 // Schedule: every CTA takes a contiguous range of the up tiles, then of the
@@ -64,7 +71,8 @@ constexpr int kCDqWarp0 = 10;
 constexpr int kCDqWarps = 16;
 constexpr int kCTable = kMaxExperts + 1;  // groups: experts and the shared one
 
-template <bool Q4, int STEPS>
+// GATHER: x by TMA gathers (tiles of up to 64 tokens)
+template <bool Q4, int STEPS, bool GATHER>
 struct CCfg {
   static constexpr int kThreads = (kCDqWarp0 + (Q4 ? kCDqWarps : 0)) * 32;
   static constexpr uint32_t kOperandCol = 256;  // TMEM: two accumulators of 128 columns, then A steps
@@ -96,6 +104,22 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, u
       "%5, %6}], [%2];" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
+}
+
+// Four rows of a map whose box is one row of 64: 4 x 128 swizzled bytes.
+__device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c, int r0, int r1,
+                                            int r2, int r3) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
+      "%4, %5, %6, %7}], [%2];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+      : "memory");
+}
+
+// Generic-proxy writes to global memory (observed through an acquire) before
+// this thread's TMA loads of them.
+__device__ __forceinline__ void fence_proxy_async_global() {
+  asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
 __device__ __forceinline__ void cp_async16_at(uint32_t dst, const void* src, uint32_t src_bytes) {
@@ -202,20 +226,23 @@ __device__ __forceinline__ float silu_mul(float g, float u) {
 }
 
 // Group table of the launch (shared memory): the groups that have tiles, in
-// order, the shared expert last.  Wave mode re-checks each slot (fail closed:
+// order, the shared expert last.  A wave's (W: WaveParams) re-checks each slot (fail closed:
 // a group whose slot does not hold the expected object and version gets no
 // tiles, and CTA 0 records the lowest such expert's status).  Every thread
 // calls it; returns the number of routed groups.
-__device__ __forceinline__ int cols_group_table(const FusedArgs& a, const WaveParams& w, bool record, int* s_mt,
+template <typename W>
+__device__ __forceinline__ int cols_group_table(const FusedArgs& a, const W& w, bool record, int* s_mt,
                                                 int* s_slot, int* s_rb, int* s_cnt, int* s_tmp) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int n = a.wave ? w.n : a.num_groups;
+  constexpr bool wave = std::is_same<W, WaveParams>::value;
+  int n = a.num_groups;
+  if constexpr (wave) n = w.n;
   int groups = 0, tiles = 0, kmin = 0x7fffffff;
   for (int i0 = 0; i0 < n; i0 += blockDim.x) {
     const int i = i0 + tid;
     int cnt = 0, slot = 0, rb = 0, code = 0, e = 0;
     if (i < n) {
-      if (a.wave) {
+      if constexpr (wave) {
         e = w.expert[i];
         cnt = __ldg(&a.counts[e]);
         rb = __ldg(&a.offsets[e]);
@@ -286,12 +313,14 @@ __device__ __forceinline__ int cols_group_table(const FusedArgs& a, const WavePa
 
 }  // namespace
 
-template <bool Q4, int STEPS>
-__global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
+template <bool Q4, int STEPS, bool GATHER, typename W>
+__global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
     fused_cols_kernel(const __grid_constant__ CUtensorMap tmW13, const __grid_constant__ CUtensorMap tmW2,
                       const __grid_constant__ CUtensorMap tmS13, const __grid_constant__ CUtensorMap tmS2,
-                      const __grid_constant__ FusedArgs a, const __grid_constant__ WaveParams w) {
-  using C = CCfg<Q4, STEPS>;
+                      const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmH,
+                      const __grid_constant__ CUtensorMap tmHS, const __grid_constant__ FusedArgs a,
+                      const __grid_constant__ W w) {
+  using C = CCfg<Q4, STEPS, GATHER>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -325,7 +354,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.ring_s; ++s) {
-      mbar_init(&sfull[s], kCTokWarps * 32 + (Q4 ? 0 : 1));
+      mbar_init(&sfull[s], kCTokWarps * (GATHER ? 1 : 32) + (Q4 ? 0 : 1));
       mbar_init(&sempty[s], 1);
     }
     for (int s = 0; s < a.ring_w; ++s) {
@@ -353,6 +382,8 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
       tma_prefetch(&tmS13);
       tma_prefetch(&tmS2);
     }
+    tma_prefetch(&tmX);
+    tma_prefetch(&tmH);
   }
   grid_wait();
   grid_release();
@@ -507,7 +538,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
         ok = wait_warp(&sfull[r.i], r.ph, abort_flag, lim);
         if (!ok) break;
         // cp.async (generic proxy) wrote the tokens: before the tensor core's reads
-        fence_proxy_async_smem();
+        if (!GATHER) fence_proxy_async_smem();
         const uint32_t w_lo = s_lo + ((r.i * stage) >> 4);
         const uint32_t bl = w_lo + (w_stage >> 4);
         if (Q4) {
@@ -646,25 +677,34 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
     }
   } else if (warp < 6 + kCTokWarps) {
     // ------------------------------------------------------------- token rows
-    const int gt = threadIdx.x - 6 * 32;  // 0..127
-    const int chunk = gt & 7;             // 16-byte chunk of a 128-byte row slice
-    const int r0 = gt >> 3;               // rows r0 + 16 i
+    const int tw = warp - 6;
+    const int gt = threadIdx.x - 6 * 32;  // copies: 16-byte chunk gt % 8 of rows gt / 8 + 16 i
+    const int chunk = gt & 7, r0 = gt >> 3;
+    constexpr int kRows = GATHER ? 1 : 8;
+    constexpr int kWarpArrivals = GATHER ? 1 : 32;
     Ring r(a.ring_s);
+    int issued = 0;  // stages
     bool ok = true;
-    // the tokens of an up tile's rows r0 + 16 i, loaded one tile ahead
-    auto tile_rows = [&](const ColsTile& t, int (&tok)[8]) {
+    // an up tile's tokens, loaded one tile ahead: of row 4 tw + 16 (lane / 4) +
+    // lane % 4 (gather; past the tile its last row's), or of rows r0 + 16 i
+    auto tile_rows = [&](const ColsTile& t, int (&tok)[kRows]) {
       if (!t.up) return;
       const int row0 = t.m * a.tile_tok;
       const int rows = min(a.tile_tok, s_cnt[t.g] - row0);
       const int* perm = a.perm + s_rb[t.g] + row0;
+      if (GATHER) {
+        const int rr = min(4 * tw + 16 * (lane >> 2) + (lane & 3), rows - 1);
+        tok[0] = t.g == g_sh ? row0 + rr : __ldg(&perm[rr]);
+      } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (16 * i >= rows) break;
-        const int rr = r0 + 16 * i;
-        tok[i] = t.g == g_sh ? row0 + rr : rr < rows ? __ldg(&perm[rr]) : 0;
+        for (int i = 0; i < kRows; ++i) {
+          if (16 * i >= rows) break;
+          const int rr = r0 + 16 * i;
+          tok[i] = t.g == g_sh ? row0 + rr : rr < rows ? __ldg(&perm[rr]) : 0;
+        }
       }
     };
-    int tok[8], tok_next[8];
+    int tok[kRows], tok_next[kRows];
     bool more = walk.next();
     if (more) tile_rows(walk.t, tok_next);
     while (more && ok) {
@@ -672,9 +712,9 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
       const bool sh = t.g == g_sh;
       const int rows = min(a.tile_tok, s_cnt[t.g] - t.m * a.tile_tok);
       const int kb_n = t.up ? a.kb_up : a.kb_dn;
-      const int n_it = (rows + 15) >> 4;  // rows past the tile's, up to the MMA's 16-column step: zero
+      const int n_it = (rows + 15) >> 4;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < kRows; ++i) {
         if (i >= n_it) break;
         tok[i] = tok_next[i];
       }
@@ -697,56 +737,92 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS>::kThreads, 1)
         ok = __shfl_sync(0xffffffffu, ok, 0);
         __syncwarp();
         if (!ok) break;
-      }
-      // row r0 + 16 i at base + (token or row) * ld
-      const __nv_bfloat16* base =
-          (t.up ? a.x : (sh ? a.hs : a.h + (size_t)s_rb[t.g] * a.h_ld) + (size_t)t.m * a.tile_tok * a.h_ld) + chunk * 8;
-      const int ld = t.up ? a.x_ld : a.h_ld;
-      const uint32_t dst0 = smem_u32(sT) + w_stage + r0 * 128 + ((chunk ^ (r0 & 7)) << 4);
-      if (n_it == 1) {  // most tiles of a short call: one row a thread
-        const uint32_t bytes = r0 < rows ? 16u : 0u;
-        const __nv_bfloat16* src = r0 < rows ? base + (size_t)(t.up ? tok[0] : r0) * ld : a.x;
+        fence_proxy_async_global();
+        // warp j loads the stage's step j in boxes of 16 rows (the last one's
+        // rows past the tile's are another group's or the tensor's zero fill:
+        // for columns that no output reads)
+        const CUtensorMap* map = sh ? &tmHS : &tmH;
+        const int row = (sh ? 0 : s_rb[t.g]) + t.m * a.tile_tok;
+        for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
+          if (!wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+          if (elect_one()) {
+            if (tw < STEPS && k0 + tw < kb_n) {
+              mbar_arrive_expect_tx(&sfull[r.i], n_it * 2048);
+              if (kWarpArrivals > 1) mbar_arrive_n(&sfull[r.i], kWarpArrivals - 1);
+              uint8_t* dst = sT + w_stage + r.i * stage + tw * b_step;
+              for (int i = 0; i < n_it; ++i)
+                tma_load_2d(dst + i * 2048, map, &sfull[r.i], (k0 + tw) * kBK, row + 16 * i);
+            } else {
+              mbar_arrive_n(&sfull[r.i], kWarpArrivals);
+            }
+          }
+          __syncwarp();
+          r.step();
+          ++issued;
+        }
+      } else if (GATHER) {
+        // quads tw, tw + 4, ... of the tile's rows, one a lane
+        const int nq = ((rows + 3) / 4 - tw + 3) / 4;
+        const int q = 4 * (lane & 7);
+        const int i0 = __shfl_sync(0xffffffffu, tok[0], q), i1 = __shfl_sync(0xffffffffu, tok[0], q + 1);
+        const int i2 = __shfl_sync(0xffffffffu, tok[0], q + 2), i3 = __shfl_sync(0xffffffffu, tok[0], q + 3);
+        const uint32_t dst0 = smem_u32(sT) + w_stage + tw * 512 + lane * 2048, bar0 = smem_u32(sfull);
+        for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
+          if (!wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+          const int ks = min(STEPS, kb_n - k0);
+          if (elect_one()) {
+            if (nq > 0) mbar_arrive_expect_tx(&sfull[r.i], ks * nq * 512);
+            else mbar_arrive(&sfull[r.i]);
+          }
+          __syncwarp();
+          if (lane < nq) {
+            uint32_t dst = dst0 + r.i * stage;
+            for (int st = 0; st < ks; ++st, dst += b_step)
+              tma_gather4(dst, &tmX, bar0 + r.i * 8, (k0 + st) * kBK, i0, i1, i2, i3);
+          }
+          __syncwarp();
+          r.step();
+          ++issued;
+        }
+      } else {
+        const __nv_bfloat16* src[kRows];
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+          if (i >= n_it) break;
+          src[i] = r0 + 16 * i < rows ? a.x + (size_t)tok[i] * a.x_ld + chunk * 8 : a.x;
+        }
+        const uint32_t dst0 = smem_u32(sT) + w_stage + r0 * 128 + ((chunk ^ (r0 & 7)) << 4);
         for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
           if (!mbar_wait(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
           const uint32_t dst = dst0 + r.i * stage;
-          cp_async16_at(dst, src, bytes);
-          cp_async16_at(dst + b_step, src + kBK, bytes);
-          if (STEPS == 4 && k0 + 2 < kb_n) {
-            cp_async16_at(dst + 2 * b_step, src + 2 * kBK, bytes);
-            cp_async16_at(dst + 3 * b_step, src + 3 * kBK, bytes);
+#pragma unroll
+          for (int i = 0; i < kRows; ++i) {
+            if (i >= n_it) break;
+            const uint32_t bytes = r0 + 16 * i < rows ? 16u : 0u;
+            cp_async16_at(dst + i * 2048, src[i], bytes);
+            cp_async16_at(dst + b_step + i * 2048, src[i] + kBK, bytes);
+            if (STEPS == 4 && k0 + 2 < kb_n) {
+              cp_async16_at(dst + 2 * b_step + i * 2048, src[i] + 2 * kBK, bytes);
+              cp_async16_at(dst + 3 * b_step + i * 2048, src[i] + 3 * kBK, bytes);
+            }
+            src[i] += STEPS * kBK;
           }
-          src += STEPS * kBK;
           cp_async_arrive_noinc(&sfull[r.i]);  // arrives when this thread's copies land
           r.step();
+          ++issued;
         }
-        continue;
-      }
-      const __nv_bfloat16* src[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (i >= n_it) break;
-        src[i] = r0 + 16 * i < rows ? base + (size_t)(t.up ? tok[i] : r0 + 16 * i) * ld : a.x;
-      }
-      for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-        if (!mbar_wait(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
-        const uint32_t dst = dst0 + r.i * stage;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (i >= n_it) break;
-          const uint32_t bytes = r0 + 16 * i < rows ? 16u : 0u;
-          cp_async16_at(dst + i * 2048, src[i], bytes);
-          cp_async16_at(dst + b_step + i * 2048, src[i] + kBK, bytes);
-          if (STEPS == 4 && k0 + 2 < kb_n) {
-            cp_async16_at(dst + 2 * b_step + i * 2048, src[i] + 2 * kBK, bytes);
-            cp_async16_at(dst + 3 * b_step + i * 2048, src[i] + 3 * kBK, bytes);
-          }
-          src[i] += STEPS * kBK;
-        }
-        cp_async_arrive_noinc(&sfull[r.i]);
-        r.step();
       }
     }
-    cp_async_wait<0>();
+    if (!GATHER) cp_async_wait<0>();
+    // on abort, the loads this warp issued land (bounded), as above
+    if (*abort_flag && lane == 0) {
+      for (int d = 0; d < a.ring_s && d < issued; ++d) {
+        const int j = issued - 1 - d;
+        const long long t0 = clock64();
+        while (!mbar_try_wait(&sfull[j % a.ring_s], (j / a.ring_s) & 1) && clock64() - t0 < kDrainCycles) {
+        }
+      }
+    }
   } else if (Q4) {
     // ------------------------------------------------------------- conversion
     const int q = warp & 3;                   // TMEM lane quarter
@@ -854,12 +930,13 @@ namespace {
 constexpr int kColsFixed = 1024 + 4096 + (4 * kCRingMax + 4 + 4 + 2) * 8 + 8 + (4 * kCTable + 1 + 96) * 4;
 constexpr int kColsSmem = 227 * 1024;
 
-template <bool Q4, int STEPS>
+template <bool Q4, int STEPS, bool GATHER, typename W>
 cudaError_t launch_cols(const CUtensorMap& tmW13, const CUtensorMap& tmW2, const CUtensorMap& tmS13,
-                        const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid, bool after,
+                        const CUtensorMap& tmS2, const CUtensorMap& tmX, const CUtensorMap& tmH,
+                        const CUtensorMap& tmHS, const FusedArgs& a, const W& w, int grid, bool after,
                         cudaStream_t s) {
   static std::atomic<unsigned long long> attr_done{0};
-  cudaError_t e = smem_attr_once(fused_cols_kernel<Q4, STEPS>, kColsSmem, attr_done);
+  cudaError_t e = smem_attr_once(fused_cols_kernel<Q4, STEPS, GATHER, W>, kColsSmem, attr_done);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
@@ -868,12 +945,12 @@ cudaError_t launch_cols(const CUtensorMap& tmW13, const CUtensorMap& tmW2, const
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(CCfg<Q4, STEPS>::kThreads, 1, 1);
+  cfg.blockDim = dim3(CCfg<Q4, STEPS, GATHER>::kThreads, 1, 1);
   cfg.dynamicSmemBytes = kColsFixed + a.ring_s * STEPS * ((Q4 ? 0 : kCSlot) + a.b_rows * 128) + a.ring_w * (kCSlot + kCScale);
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = after ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, fused_cols_kernel<Q4, STEPS>, tmW13, tmW2, tmS13, tmS2, a, w);
+  return cudaLaunchKernelEx(&cfg, fused_cols_kernel<Q4, STEPS, GATHER, W>, tmW13, tmW2, tmS13, tmS2, tmX, tmH, tmHS, a, w);
 }
 
 }  // namespace
@@ -882,9 +959,11 @@ cudaError_t launch_cols(const CUtensorMap& tmW13, const CUtensorMap& tmW2, const
 // of a call of T tokens.  A tile of as few tokens as most experts have leaves
 // room for more stages of more K each; a group with more rows takes several
 // tiles (and converts or reads its weights for each).  4-bit: at least as many
-// stages as the TMEM ring holds, the rest of shared memory to codes in flight.
+// stages as the TMEM ring holds, the rest of shared memory to codes in flight;
+// from 24 rows a group on 128-token tiles (the call at 1,600 tokens, 31 rows a
+// group, 406 us against 426 with 64; at 1,200 388 both).
 int cols_tile_tokens(long long rows, int groups) {
-  return rows <= 10LL * groups ? 32 : rows <= 32LL * groups ? 64 : 128;
+  return rows <= 10LL * groups ? 32 : rows <= 24LL * groups ? 64 : 128;
 }
 
 void cols_rings(FusedArgs& a, bool q4, int T) {
@@ -904,12 +983,19 @@ void cols_rings(FusedArgs& a, bool q4, int T) {
 }
 
 cudaError_t launch_fused_cols(bool q4, const CUtensorMap& tmW13, const CUtensorMap& tmW2, const CUtensorMap& tmS13,
-                              const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid,
-                              bool after, cudaStream_t s) {
+                              const CUtensorMap& tmS2, const CUtensorMap& tmX, const CUtensorMap& tmH,
+                              const CUtensorMap& tmHS, const FusedArgs& a, const WaveParams& w, int grid, bool after,
+                              cudaStream_t s) {
   if (grid < 1) return cudaSuccess;
-  if (q4) return launch_cols<true, 4>(tmW13, tmW2, tmS13, tmS2, a, w, grid, after, s);
-  return a.steps == 4 ? launch_cols<false, 4>(tmW13, tmW2, tmS13, tmS2, a, w, grid, after, s)
-                      : launch_cols<false, 2>(tmW13, tmW2, tmS13, tmS2, a, w, grid, after, s);
+  const auto go = [&](auto launch, const auto& wave) {
+    return launch(tmW13, tmW2, tmS13, tmS2, tmX, tmH, tmHS, a, wave, grid, after, s);
+  };
+  if (!q4)
+    return a.steps == 4 ? go(launch_cols<false, 4, true, NoWave>, NoWave{})
+                        : go(launch_cols<false, 2, true, NoWave>, NoWave{});
+  if (a.tile_tok > 64)
+    return a.wave ? go(launch_cols<true, 4, false, WaveParams>, w) : go(launch_cols<true, 4, false, NoWave>, NoWave{});
+  return a.wave ? go(launch_cols<true, 4, true, WaveParams>, w) : go(launch_cols<true, 4, true, NoWave>, NoWave{});
 }
 
 }  // namespace msi

@@ -6,6 +6,7 @@
 #pragma once
 
 #include <atomic>
+#include <type_traits>
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -134,6 +135,13 @@ struct WaveParams {
   unsigned long long expected[kMaxWave];
 };
 
+// In its place in gemm_cols.cu's resident launches (with its seven tensor maps
+// and WaveParams a launch has 5.4 KB of parameters, and a one-token call took
+// 57 us; without WaveParams 53, as with four maps and WaveParams).
+struct NoWave {
+  int none;
+};
+
 // One wave's gate-up and down projections in one launch (gemm_fused.cu).
 struct FusedArgs {
   const Group* groups;
@@ -217,8 +225,9 @@ cudaError_t launch_fused_wave_pair_q4(const CUtensorMap& tmQ13, const CUtensorMa
 int cols_tile_tokens(long long rows, int groups);
 void cols_rings(FusedArgs& a, bool q4, int T);
 cudaError_t launch_fused_cols(bool q4, const CUtensorMap& tmW13, const CUtensorMap& tmW2, const CUtensorMap& tmS13,
-                              const CUtensorMap& tmS2, const FusedArgs& a, const WaveParams& w, int grid,
-                              bool after, cudaStream_t s);
+                              const CUtensorMap& tmS2, const CUtensorMap& tmX, const CUtensorMap& tmH,
+                              const CUtensorMap& tmHS, const FusedArgs& a, const WaveParams& w, int grid, bool after,
+                              cudaStream_t s);
 
 // GEMM tiling
 constexpr int kBM = 128;

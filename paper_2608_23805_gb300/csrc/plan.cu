@@ -695,6 +695,8 @@ struct FwdCtx {
   int stall;  // MSI_FAULT_DEVICE_WAIT armed for this call
   cudaStream_t cs;
   CUtensorMap tm_h, tm_x, tm_hs;
+  CUtensorMap tm_x1, tm_h16, tm_hs16;  // gemm_cols.cu's, from its first launch on
+  bool cols_maps = false;
   // host-buffer calls: the rows land on the copy stream (x_ready, recorded
   // there); the route ids and the output rows go back on it
   cudaStream_t io = nullptr;
@@ -737,9 +739,9 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 
 // Weights as MMA rows (gemm_cols.cu), in one launch with a resident call's
 // shared expert, while the groups average few rows:
-//   4-bit: at 8, 250 and 4,096 tokens of the Qwen-shaped layer 65, 300 and 432
+//   4-bit: at 8, 250 and 4,096 tokens of the Qwen-shaped layer 62, 288 and 416
 //     us against 91, 534 and 546 in two row-major launches; the call at 8,192
-//     tokens 990 against 1,209, at 20,000 (390 rows a group, four tiles and
+//     tokens 964 against 1,209, at 20,000 (390 rows a group, four tiles and
 //     conversions) 2,105 against 2,215, at 32,768 3,508 against 3,086 on pairs.
 //     A wave up to 256 rows.
 //   bf16: where the launches' latency is what counts (one token: 24 us for
@@ -914,7 +916,8 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
   }
   const int nb = (f.T + L.tm - 1) / L.tm;
   if (!make_tmap(&f.tm_x, f.x, H, f.T, 128)) return MSI_ERR_CUDA;
-  if (d.has_shared) {
+  const bool cols = tp.E > 0 && cols_tiles(p, f, (long long)f.T * k, E);  // the row-major kernels' maps are not needed
+  if (d.has_shared && !cols) {
     if (!make_tmap(&f.tm_hs, at<char>(ws, L.hs), I, f.T, 128)) return MSI_ERR_CUDA;
   }
   // up to kScatterWarps router blocks: one scatter block covers them all and
@@ -948,7 +951,7 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
     xa.tab_slot = at<int>(ws, L.table);
     xa.tab_expected = at<unsigned long long>(ws, L.expected);
     xa.layer = tp.layer;
-    if (fused_resident(p, f, (long long)f.T * k, E) || cols_tiles(p, f, (long long)f.T * k, E)) {
+    if (fused_resident(p, f, (long long)f.T * k, E) || cols) {
       xa.ready = at<int>(ws, L.ready);
       xa.n_ready = ready_bank(f);
     }
@@ -972,7 +975,7 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
     CK(cudaStreamWaitEvent(f.io, p->ev_io_a, 0));
     CK(cudaMemcpyAsync(f.ids_host, f.ev->ids, Tk * sizeof(int32_t), cudaMemcpyDeviceToHost, f.io));
   }
-  if (!make_tmap(&f.tm_h, at<char>(ws, L.h), I, Tk, 128)) return MSI_ERR_CUDA;
+  if (!cols && !make_tmap(&f.tm_h, at<char>(ws, L.h), I, Tk, 128)) return MSI_ERR_CUDA;
   return MSI_OK;
 }
 
@@ -1125,10 +1128,19 @@ msi_status routed_ffn(msi_plan* p, FwdCtx& f, int ng, int grid1, int grid2, long
         all += (long long)((f.T + fa.tile_tok - 1) / fa.tile_tok) * (fa.nt_up + fa.nt_dn);
       }
       cols_rings(fa, !bf16, f.T);
+      // the tokens by TMA: x a gather of four rows, h in boxes of 16
+      if (!f.cols_maps) {
+        if (!make_tmap(&f.tm_x1, fa.x, d.hidden, f.T, 1) ||
+            !make_tmap(&f.tm_h16, fa.h, d.inter, (uint64_t)f.T * d.top_k, 16) ||
+            (fa.sh_rows > 0 && !make_tmap(&f.tm_hs16, fa.hs, d.inter, f.T, 16)))
+          return MSI_ERR_CUDA;
+        if (fa.sh_rows == 0) f.tm_hs16 = f.tm_h16;
+        f.cols_maps = true;
+      }
       const int grid = (int)std::min<long long>(p->sms - spare, std::max<long long>(1, all));
       LAUNCH(p, MSI_K_FFN, f.cs,
              launch_fused_cols(!bf16, p->tm_p13, bf16 ? p->tm_w2 : p->tm_c2, d.has_shared ? p->tm_psh13 : p->tm_p13,
-                               d.has_shared ? p->tm_sh2 : p->tm_p13, fa, wv, grid, wp == nullptr, f.cs));
+                               d.has_shared ? p->tm_sh2 : p->tm_p13, f.tm_x1, f.tm_h16, f.tm_hs16, fa, wv, grid, wp == nullptr, f.cs));
       return MSI_OK;
     }
     if (!bf16) {
