@@ -374,7 +374,7 @@ WsLayout layout(const msi_plan* p, int T) {
   L.total = take(12);     // 128-row tiles, 256-row pair tiles; the router selection's ticket
   L.sh_group = take(sizeof(Group));
   L.sh_total = take(8);
-    // the tensor router's logits (a longer call's go to the GEMMs' buffers, or
+  // the tensor router's logits (a longer call's go to the GEMMs' buffers, or
   // through here in row chunks): at least 1.5 H rows
   if (tensor_router(p->d)) {
     L.logits_bytes = 3 * E * H * 2 + 8 * (size_t)T * std::max<size_t>(1, E / 128) * std::min<size_t>(k + 1, E);
