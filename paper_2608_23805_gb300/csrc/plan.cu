@@ -747,8 +747,8 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 //   bf16: where the launches' latency is what counts (one token: 24 us for
 //     what took 28 + 25 on a side stream).  From some 40 tokens on both
 //     orientations stream the weights at the same rate (0.97 of HBM), and the
-//     row-major tiles read the tokens half as often (the call at 250 tokens 524
-//     in both, at 600 545 row-major, 555 here).  Not a wave: its launch has no
+//     row-major tiles read the tokens half as often (the call at 300 tokens 532
+//     in both, at 600 541 row-major and 543 here, at 2,000 581 and 607).  Not a wave: its launch has no
 //     shared expert to take in.
 constexpr long long kColsMaxRows = 512, kColsMaxRowsWave = 256, kColsMaxRowsBf16 = 8;
 bool cols_tiles(const msi_plan* p, const FwdCtx& f, long long rows, int ng, bool wave = false) {
