@@ -40,10 +40,8 @@ struct RouterTcArgs {
   int T, H, E, k;
   int chunk;               // experts per logits CTA (16, 32, 64 or 128; divides E)
   int nchunk;              // E / chunk
-  int ksplit;              // parts of K, each its own CTA (1, 2 or 4)
-  int stack;               // planes stacked along the MMA's N (router_tc.cu)
   int t0, rows;            // the launch's tokens [t0, t0 + rows), t0 a multiple of 128
-  float* logits;           // [ksplit, rows, E] partial sums (scratch)
+  float* logits;           // [rows, E] (scratch)
   int* ids;                // [T, k]
   float* weights;          // [T, k]
   float* gap;              // [T] or nullptr
@@ -62,13 +60,7 @@ struct RouterTcArgs {
   int stall;               // as GemmArgs::stall
 };
 
-// How the logits of a call's rows are cut into CTAs.
-struct RouterSplit {
-  int chunk, ksplit;
-  bool stack;
-};
-constexpr int kSplitTokens = 64;  // longest call with K parts and stacked planes (router_tc.cu)
-RouterSplit router_split(int T, int E, int sms);
+int router_chunk(int T, int E, int sms);
 
 struct ScanArgs {
   const int* bcount;

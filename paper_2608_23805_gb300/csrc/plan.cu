@@ -812,12 +812,8 @@ msi_status route_rows(msi_plan* p, FwdCtx& f, const float* rw, const msi_route_e
       ra.logits = at<float>(ws, L.h);
     }
     const int chunk_rows = cap / row >= (size_t)f.T ? f.T : (int)(cap / row / 128 * 128);
-    const RouterSplit sp = router_split(chunk_rows, E, p->sms);
-    ra.chunk = sp.chunk;
-    ra.nchunk = E / sp.chunk;
-    ra.ksplit = sp.ksplit;
-    ra.stack = router_split(f.T, E, p->sms).stack;
-    while (ra.ksplit > 1 && ra.ksplit * row * (size_t)chunk_rows > cap) ra.ksplit /= 2;
+    ra.chunk = router_chunk(chunk_rows, E, p->sms);
+    ra.nchunk = E / ra.chunk;
     const bool fuse = first && xa != nullptr && f.T <= kFuseTokens;
     // a long resident call begins with a kernel of its own, so that the side
     // stream's shared expert runs beside the logits and not after them

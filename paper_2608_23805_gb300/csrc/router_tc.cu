@@ -15,19 +15,18 @@
 // an fp32 GEMM up to accumulation order.
 //
 // Two kernels:
-//  1. router_logits_kernel, one CTA per (128 tokens, CH experts, K split):
-//     eight warps read the chunk's fp32 weights, split them and write the
-//     three planes as swizzled operand tiles; x tiles come by TMA; 12 MMAs per
-//     64 of K; the logits (of the CTA's part of K) go to global memory, where
-//     the next kernel finds them in L2.
+//  1. router_logits_kernel, one CTA per (128 tokens, CH experts): sixteen
+//     warps read the chunk's fp32 weights, split them and write the three
+//     planes as swizzled operand tiles; x tiles come by TMA; 12 MMAs per 64 of
+//     K; the logits go to global memory, where the next kernel finds them in
+//     L2.  A logit is one accumulation chain over K whatever the call's length
+//     and cut: a row's route event does not depend on the rows beside it.
 //     What bounds it: the operand feed (x tile and weights, 48 KB per 64 of K
 //     at CH = 128, at the SM's 64 bytes a cycle from L2) for long calls, and
-//     the latency of one CTA's pass over K for short ones (the two launches
-//     took 40 us for one token as 4 CTAs, and take 17 as 128).  So short calls
-//     are cut into smaller expert chunks, then over K, until the grid fills
-//     the SMs (router_split).
-//  2. router_select_kernel, one warp per token: sums the K parts, selects the
-//     top k + 1, weights, gap, the 32-token block's expert histogram and the
+//     the latency of one CTA's pass over K for short ones (one token: 24 us as
+//     4 CTAs of 128 experts, 16 as 32 of 16).  So short calls are cut into
+//     smaller expert chunks (router_chunk).
+//  2. router_select_kernel, one warp per token: selects the top k + 1, weights, gap, the 32-token block's expert histogram and the
 //     shared-expert gate sigmoid(x . w_sg).  A call of at most kFuseTokens
 //     tokens also does the scatter's work here (offsets, permutation,
 //     generation re-check, GEMM groups), in the CTA that finishes last.
@@ -41,10 +40,7 @@ constexpr int kCvtWarps = 16;                      // weight split, then the epi
 constexpr int kRlThreads = (kCvtWarps + 2) * 32;   // + TMA producer, MMA issuer
 constexpr int kXBytes = 128 * 64 * 2;              // x tile (64 of K)
 
-// STACK: the three planes are one MMA operand of 3 CH rows (two of 192 at
-// CH = 128) with an accumulator each, summed at the end: 4 or 8 MMAs per 64 of
-// K instead of 12 (an MMA of up to 96 columns takes 48 cycles, of 128 64).
-template <int CH, bool STACK>
+template <int CH>
 struct RlCfg {
   static constexpr int kPlane = CH * 128;          // one plane's rows (64 of K)
   static constexpr int kStage = kXBytes + 3 * kPlane;
@@ -60,9 +56,7 @@ struct RlCfg {
   static constexpr int kGroupWarps = kCvtWarps / kGroups;
   static constexpr int kVec = CH * 16 / (kGroupWarps * 32);  // 16-byte loads per thread and stage
   static_assert(kGroups <= kStages && kVec * kGroupWarps * 32 == CH * 16, "weight groups");
-  static constexpr int kAcc = STACK ? 3 : 1;       // accumulators of CH columns
-  static constexpr int kCols = CH * kAcc <= 32 ? 32 : CH * kAcc <= 64 ? 64 : CH * kAcc <= 128 ? 128
-                               : CH * kAcc <= 256 ? 256 : 512;  // TMEM columns
+  static constexpr int kCols = CH <= 32 ? 32 : CH;  // TMEM columns
 };
 
 // hi, mid and lo planes of two weights, as packed bf16 pairs
@@ -73,14 +67,13 @@ __device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t&
   lo = pack_bf16x2(a1 - bf16_lo(mid), b1 - bf16_hi(mid));
 }
 
-// The weight warps' loop: the chunk's fp32 rows (src: its first row at the
-// CTA's first K; H apart), 64 of K per stage, into the three planes of the
-// stage.  ALIGNED: src is 16-byte aligned.
-template <int CH, bool STACK, bool ALIGNED>
+// The weight warps' loop: the chunk's fp32 rows (src: its first row; H apart),
+// 64 of K per stage, into the three planes of the stage.  ALIGNED: src is 16-byte aligned.
+template <int CH, bool ALIGNED>
 __device__ __forceinline__ void split_weights(const float* src, int H, int nstage, uint8_t* smem,
                                               uint64_t* full, uint64_t* empty, volatile int* abort_flag,
                                               long long lim) {
-  using C = RlCfg<CH, STACK>;
+  using C = RlCfg<CH>;
   // thread: 16-byte piece of the rows row + 2 * kGroupWarps * i of the chunk
   const int group = (threadIdx.x >> 5) / C::kGroupWarps;
   const int gt = threadIdx.x - group * C::kGroupWarps * 32;
@@ -121,11 +114,11 @@ __device__ __forceinline__ void split_weights(const float* src, int H, int nstag
   }
 }
 
-template <int CH, bool STACK>
+template <int CH>
 __global__ void __launch_bounds__(kRlThreads, 1)
     router_logits_kernel(const __grid_constant__ CUtensorMap tmX, const RouterTcArgs a,
                          const __grid_constant__ TableParams tp) {
-  using C = RlCfg<CH, STACK>;
+  using C = RlCfg<CH>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -140,13 +133,9 @@ __global__ void __launch_bounds__(kRlThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // the chunks of one token tile are neighbours in launch order, so the x
   // tile is read from HBM once and from L2 by the other chunks
-  int b = blockIdx.x;
-  const int c = b % a.nchunk;
-  b /= a.nchunk;
-  const int part = b % a.ksplit;
-  const int m0 = a.t0 + b / a.ksplit * 128;
-  const int nstage = a.H / 64 / a.ksplit;
-  const int kb0 = part * nstage;
+  const int c = blockIdx.x % a.nchunk;
+  const int m0 = a.t0 + blockIdx.x / a.nchunk * 128;
+  const int nstage = a.H / 64;
   const long long lim = a.wait_limit;
 
   if (tid == 0) {
@@ -191,7 +180,7 @@ __global__ void __launch_bounds__(kRlThreads, 1)
         const int s = it % C::kStages;
         if (!mbar_wait(&empty[s], ((it / C::kStages) & 1) ^ 1, abort_flag, lim)) break;
         mbar_arrive_expect_tx(&full[s], kXBytes);
-        tma_load_2d(smem + s * C::kStage, &tmX, &full[s], (kb0 + it) * 64, m0);
+        tma_load_2d(smem + s * C::kStage, &tmX, &full[s], it * 64, m0);
       }
       // on abort the armed loads land before shared memory is released (a
       // stage's barrier may still lack the weight arrivals: bounded)
@@ -217,23 +206,12 @@ __global__ void __launch_bounds__(kRlThreads, 1)
       const uint32_t st = smem_u32(smem + s * C::kStage);
       const uint64_t ad = sw128_desc(st);
       if (elect_one()) {
-        if (STACK) {
-          constexpr int kN = CH == 128 ? 192 : 3 * CH;  // rows per MMA
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
+        for (int plane = 0; plane < 3; ++plane) {
+          const uint64_t bd = sw128_desc(st + kXBytes + plane * C::kPlane);
 #pragma unroll
-            for (int n0 = 0; n0 < 3 * CH; n0 += kN)
-              umma_bf16(tm + n0, ad + 2 * kk, sw128_desc(st + kXBytes + n0 * 128) + 2 * kk, idesc_bf16(128, kN),
-                        (it | kk) != 0);
-          }
-        } else {
-#pragma unroll
-          for (int plane = 0; plane < 3; ++plane) {
-            const uint64_t bd = sw128_desc(st + kXBytes + plane * C::kPlane);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              umma_bf16(tm, ad + 2 * kk, bd + 2 * kk, idesc_bf16(128, CH), (it | plane | kk) != 0);
-          }
+          for (int kk = 0; kk < 4; ++kk)
+            umma_bf16(tm, ad + 2 * kk, bd + 2 * kk, idesc_bf16(128, CH), (it | plane | kk) != 0);
         }
         umma_commit(&empty[s]);
       }
@@ -253,11 +231,11 @@ __global__ void __launch_bounds__(kRlThreads, 1)
     }
   } else {
     // ------------------------------------------------------------- weights
-    const float* src = a.wr + (size_t)c * CH * a.H + (size_t)kb0 * 64;
+    const float* src = a.wr + (size_t)c * CH * a.H;
     if ((reinterpret_cast<uintptr_t>(a.wr) & 15) == 0)
-      split_weights<CH, STACK, true>(src, a.H, nstage, smem, full, empty, abort_flag, lim);
+      split_weights<CH, true>(src, a.H, nstage, smem, full, empty, abort_flag, lim);
     else
-      split_weights<CH, STACK, false>(src, a.H, nstage, smem, full, empty, abort_flag, lim);
+      split_weights<CH, false>(src, a.H, nstage, smem, full, empty, abort_flag, lim);
     // ------------------------------------------------------------- logits out
     if (a.stall && tid == 0) mbar_wait(never, 0, abort_flag, lim);  // runs out: abort
     const bool ready = __all_sync(0xffffffffu, mbar_wait(tfull, 0, abort_flag, lim)) && !*abort_flag;
@@ -268,22 +246,12 @@ __global__ void __launch_bounds__(kRlThreads, 1)
     const int c0 = (warp >> 2) * kPer;
     if (ready && c0 < CH) {
       const uint32_t tb = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + c0;
-      float* dst = a.logits + ((size_t)part * a.rows + (t - a.t0)) * a.E + c * CH + c0;
+      float* dst = a.logits + (size_t)(t - a.t0) * a.E + c * CH + c0;
 #pragma unroll
       for (int e0 = 0; e0 < kPer; e0 += 16) {
         uint32_t r[16];
         tmem_ld16(tb + e0, r);
         tmem_ld_wait(r);
-        if (STACK) {
-          uint32_t mid[16], lo[16];
-          tmem_ld16(tb + CH + e0, mid);
-          tmem_ld16(tb + 2 * CH + e0, lo);
-          tmem_ld_wait(mid);
-          tmem_ld_wait(lo);
-#pragma unroll
-          for (int i = 0; i < 16; ++i)
-            r[i] = __float_as_uint(__uint_as_float(r[i]) + (__uint_as_float(mid[i]) + __uint_as_float(lo[i])));
-        }
         if (t < a.T && t < a.t0 + a.rows) {
           st_global_v8(dst + e0, r);
           st_global_v8(dst + e0 + 8, r + 8);
@@ -337,33 +305,12 @@ struct SelectScratch {     // shared memory of one warp
 template <int NV>
 __device__ __forceinline__ int select_token(const RouterTcArgs& a, int t, int lane, SelectScratch& sc) {
   const int E = a.E, k = a.k;
-  const size_t part_stride = (size_t)a.rows * E;
   const float* L = a.logits + (size_t)(t - a.t0) * E;
   float4 v[NV];
-  auto load = [&](const float* P, float4 (&d)[NV]) {
 #pragma unroll
-    for (int i = 0; i < NV; ++i)
-      d[i] = 128 * i + 4 * lane < E ? *reinterpret_cast<const float4*>(P + 128 * i + 4 * lane)
-                                    : make_float4(0.f, 0.f, 0.f, 0.f);
-  };
-  // the K parts in a fixed order: p0 + p1 + (p2 + p3)
-  load(L, v);
-  if (a.ksplit >= 2) {
-    float4 p1[NV], p2[NV], p3[NV];
-    load(L + part_stride, p1);
-    if (a.ksplit == 4) {
-      load(L + 2 * part_stride, p2);
-      load(L + 3 * part_stride, p3);
-    }
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      v[i].x += p1[i].x; v[i].y += p1[i].y; v[i].z += p1[i].z; v[i].w += p1[i].w;
-      if (a.ksplit == 4) {
-        v[i].x += p2[i].x + p3[i].x; v[i].y += p2[i].y + p3[i].y;
-        v[i].z += p2[i].z + p3[i].z; v[i].w += p2[i].w + p3[i].w;
-      }
-    }
-  }
+  for (int i = 0; i < NV; ++i)
+    v[i] = 128 * i + 4 * lane < E ? *reinterpret_cast<const float4*>(L + 128 * i + 4 * lane)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
   uint32_t key[4 * NV], hk = 0u;
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
@@ -410,10 +357,7 @@ __device__ __forceinline__ int select_token(const RouterTcArgs& a, int t, int la
       const int q = u + lane;
       if (q < n) {
         const int e = sc.id[q];
-        float x = L[e];
-        if (a.ksplit >= 2) x += L[part_stride + e];
-        if (a.ksplit == 4) x += L[2 * part_stride + e] + L[3 * part_stride + e];
-        sc.word[q] = entry_word(logit_key(x), e);
+        sc.word[q] = entry_word(logit_key(L[e]), e);
       }
     }
     __syncwarp();
@@ -551,14 +495,14 @@ __global__ void __launch_bounds__(512, 2) router_select_scatter_kernel(const Rou
   scatter_call(a.ids, a.T, a.k, a.E, s, s.tab_slot != nullptr, slot, code, sh);
 }
 
-template <int CH, bool STACK>
+template <int CH>
 cudaError_t launch_logits(const CUtensorMap& tmX, const RouterTcArgs& a, const TableParams& tp, cudaStream_t s) {
   static std::atomic<unsigned long long> attr_done{0};
-  constexpr int smem = RlCfg<CH, STACK>::kSmem;
-  cudaError_t e = smem_attr_once(router_logits_kernel<CH, STACK>, smem, attr_done);
+  constexpr int smem = RlCfg<CH>::kSmem;
+  cudaError_t e = smem_attr_once(router_logits_kernel<CH>, smem, attr_done);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)((a.rows + 127) / 128) * a.nchunk * a.ksplit;
-  router_logits_kernel<CH, STACK><<<grid, kRlThreads, smem, s>>>(tmX, a, tp);
+  const unsigned grid = (unsigned)((a.rows + 127) / 128) * a.nchunk;
+  router_logits_kernel<CH><<<grid, kRlThreads, smem, s>>>(tmX, a, tp);
   return cudaGetLastError();
 }
 
@@ -570,40 +514,32 @@ cudaError_t select_nv(const RouterTcArgs& a, const ScatterArgs* sa, cudaStream_t
 
 }  // namespace
 
-// Expert chunk and K split of a call of T rows: the cut with the least time by
-// a fit of the measured launches (event-timed over 1 to 8,192 rows, 512
-// experts, H 2,048, every chunk and split): about 6 us a CTA, then 0.25 us +
-// 2 ns per expert of its chunk for each 64 of K, per round of CTAs on the SMs.
-// One token: 16 experts x 4 parts 7.0 us (128 experts, one part: 24).
-// K parts and stacked planes sum a logit in another order than one chain over
-// K.  That moves it by about 1e-6, enough to swap a pair of experts that close
-// on one row in some ten thousand, so it is done where latency is all there is
-// (up to kSplitTokens) and every longer call keeps the one chain.
-RouterSplit router_split(int T, int E, int sms) {
+// Experts per logits CTA of a call of T rows: the cut with the least time by a
+// fit of the measured launches (event-timed over 1 to 8,192 rows, 512 experts,
+// H 2,048, every chunk): about 6 us a CTA, then 0.25 us + 2 ns per expert of
+// its chunk for each 64 of K, per round of CTAs on the SMs.
+int router_chunk(int T, int E, int sms) {
   const int mt = (T + 127) / 128;
-  const bool split = T <= kSplitTokens;
-  RouterSplit best{16, 1, split};
+  int best = 16;
   double cost = 1e30;
-  for (int ch = 16; ch <= 128 && E % ch == 0; ch *= 2)
-    for (int ks = 1; ks <= (split ? 4 : 1); ks *= 2) {
-      const int waves = (int)(((long long)mt * (E / ch) * ks + sms - 1) / sms);
-      const double c = waves * (6.0 + 32.0 / ks * (0.25 + ch * 0.002)) + 0.5 * ks;
-      if (c < cost) {
-        cost = c;
-        best.chunk = ch;
-        best.ksplit = ks;
-      }
+  for (int ch = 16; ch <= 128 && E % ch == 0; ch *= 2) {
+    const int waves = (int)(((long long)mt * (E / ch) + sms - 1) / sms);
+    const double c = waves * (6.0 + 32.0 * (0.25 + ch * 0.002));
+    if (c < cost) {
+      cost = c;
+      best = ch;
     }
+  }
   return best;
 }
 
 cudaError_t launch_router_logits(const CUtensorMap& tmX, const RouterTcArgs& a, const TableParams& tp,
                                  cudaStream_t s) {
   switch (a.chunk) {
-    case 16: return a.stack ? launch_logits<16, true>(tmX, a, tp, s) : launch_logits<16, false>(tmX, a, tp, s);
-    case 32: return a.stack ? launch_logits<32, true>(tmX, a, tp, s) : launch_logits<32, false>(tmX, a, tp, s);
-    case 64: return a.stack ? launch_logits<64, true>(tmX, a, tp, s) : launch_logits<64, false>(tmX, a, tp, s);
-    default: return a.stack ? launch_logits<128, true>(tmX, a, tp, s) : launch_logits<128, false>(tmX, a, tp, s);
+    case 16: return launch_logits<16>(tmX, a, tp, s);
+    case 32: return launch_logits<32>(tmX, a, tp, s);
+    case 64: return launch_logits<64>(tmX, a, tp, s);
+    default: return launch_logits<128>(tmX, a, tp, s);
   }
 }
 

@@ -1,6 +1,6 @@
 """The tensor router's route events over the sizes at which its launches
-change: expert chunks and K parts (few to many 128-row tiles, 16 to 512
-experts), selection with and without the scatter, row chunks through a small
+change: expert chunks (few to many 128-row tiles, 16 to 512 experts),
+selection with and without the scatter, row chunks through a small
 scratch, misaligned router weights, exact ties, and rows whose top experts
 share few lanes of the selecting warp.
 
@@ -82,6 +82,18 @@ def test_shapes(T, E, k, H):
     # (512, 1, 256) at 5,000 rows: the logits' scratch holds fewer rows than the call
     x, wr = inputs(T, E, H, 1)
     check(x, wr, k, route(x, wr, E, k, H))
+
+
+@pytest.mark.parametrize("E,k,H", [(512, 10, 2048), (128, 8, 256), (48, 4, 1024)])
+def test_event_does_not_depend_on_the_call(E, k, H):
+    # a row decoded alone, in a small batch and in a prefill: the same bits
+    x, wr = inputs(300, E, H, 6)
+    whole = route(x, wr, E, k, H)
+    for T in (1, 7, 33, 64, 65, 128, 257):
+        ids, w, _, gap = route(x[:T], wr, E, k, H)
+        assert (ids == whole[0][:T]).all()
+        assert (w.view(np.uint32) == whole[1][:T].view(np.uint32)).all()
+        assert (gap.view(np.uint32) == whole[3][:T].view(np.uint32)).all()
 
 
 @pytest.mark.parametrize("T", [5, 700])
