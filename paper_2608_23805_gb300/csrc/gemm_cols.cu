@@ -206,6 +206,67 @@ __device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
 
+// A conversion warp's waits, conversions and arrivals (ColsConvert).
+struct ConvertOps {
+  uint64_t *wfull, *wempty, *sempty, *afull;  // afull: the set's
+  volatile int* abort_flag;
+  const FusedArgs& a;  // 4-bit rings are powers of two
+  uint32_t half, sw, ss, dst, x0, x[4];
+  int lane, at;
+
+  __device__ __forceinline__ bool slot(uint32_t w) const {
+    return wait_warp(&wfull[w & (a.ring_w - 1)], (w & a.ring_w) != 0, abort_flag, a.wait_limit);
+  }
+  __device__ __forceinline__ bool stage(uint32_t st) const {
+    return st < 2 || wait_warp(&sempty[(st - 2) & (a.ring_s - 1)], ((st - 2) & a.ring_s) != 0, abort_flag, a.wait_limit);
+  }
+  __device__ __forceinline__ void codes(uint32_t w, bool any) const {
+    const uint32_t wi = w & (a.ring_w - 1);
+    if (any) {
+      tc_fence_after();
+      // half a slot: 128 codes and four scales of the row
+      const uint32_t src = sw + wi * kCSlot + at * 128 + ((half << 6) ^ x0);
+      const uint2 sc = ld_shared_v2(ss + wi * kCScale + at * 16 + half * 8);
+      const uint4 c0 = ld_shared_v4(src + x[0]), c1 = ld_shared_v4(src + x[1]);
+      convert32(c0, sc.x & 0xFFFFu, dst);
+      const uint4 c2 = ld_shared_v4(src + x[2]);
+      convert32(c1, sc.x >> 16, dst + 16);
+      const uint4 c3 = ld_shared_v4(src + x[3]);
+      convert32(c2, sc.y & 0xFFFFu, dst + 32);
+      convert32(c3, sc.y >> 16, dst + 48);
+      tmem_st_wait();
+      tc_fence_before();
+    }
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive(afull);
+      mbar_arrive_n(&wempty[wi], 2);  // the warp's rows of the slot are consumed, for two sets
+    }
+  }
+  __device__ __forceinline__ void rows(uint32_t w, uint32_t j) const {
+    tc_fence_after();
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const uint32_t src = sw + (w & (a.ring_w - 1)) * kCSlot + at * 128 + ((p << 6) ^ x0);
+      const uint4 b0 = ld_shared_v4(src + x[0]), b1 = ld_shared_v4(src + x[1]);
+      const uint4 b2 = ld_shared_v4(src + x[2]), b3 = ld_shared_v4(src + x[3]);
+      const uint32_t o[16] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w,
+                              b2.x, b2.y, b2.z, b2.w, b3.x, b3.y, b3.z, b3.w};
+      tmem_st16(dst + j * 32 + 16 * p, o);
+    }
+    tmem_st_wait();
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0 && j) mbar_arrive(afull);
+  }
+  __device__ __forceinline__ void none() const {
+    if (lane == 0) mbar_arrive(afull);
+  }
+  __device__ __forceinline__ void pass(uint32_t w) const {
+    if (lane == 0) mbar_arrive(&wempty[w & (a.ring_w - 1)]);
+  }
+};
+
 __device__ __forceinline__ void st_shared_u16(uint32_t addr, uint32_t v) {
   asm volatile("{\n\t.reg .b16 h;\n\tcvt.u16.u32 h, %1;\n\tst.shared.b16 [%0], h;\n\t}" ::"r"(addr), "r"(v)
                : "memory");
@@ -826,92 +887,24 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
   } else if (Q4) {
     // ------------------------------------------------------------- conversion
     const int q = warp & 3;                   // TMEM lane quarter
-    // half stages set, set + 4, ... of the CTA's sequence: half set & 1 of the
-    // stages of parity set >> 1
-    const int set = (warp - kCDqWarp0) >> 2;
-    const uint32_t odd = set >> 1, half = set & 1;
-    const uint32_t s_mask = a.ring_s - 1, s_log = 31 - __clz(a.ring_s);
-    const uint32_t w_mask = a.ring_w - 1, w_log = 31 - __clz(a.ring_w);
+    const uint32_t set = (warp - kCDqWarp0) >> 2;
+    ColsConvert conv(set);
+    ConvertOps op{wfull, wempty, sempty, afull + set, abort_flag, a};
+    op.lane = lane;
+    op.half = conv.half;
+    op.sw = smem_u32(sW);
+    op.ss = smem_u32(sS);
+    op.dst = tmem_base + ((uint32_t)(q * 32) << 16) + C::kOperandCol + set * 64;
     // the thread's row in a slot: down tiles in order, up tiles 64 gate rows,
     // then 64 up rows; 16-byte chunk c of row r lies at chunk c ^ (r & 7)
     const int at_dn = q * 32 + lane, at_up = (lane >> 4) * 64 + q * 16 + (lane & 15);
-    const uint32_t x0 = (lane & 4) << 4;
-    const uint32_t x[4] = {(lane & 3u) << 4, (1u ^ (lane & 3u)) << 4, (2u ^ (lane & 3u)) << 4, (3u ^ (lane & 3u)) << 4};
-    const uint32_t sw0 = smem_u32(sW), ss0 = smem_u32(sS);
-    const uint32_t tdst = tmem_base + ((uint32_t)(q * 32) << 16) + C::kOperandCol;
-    uint32_t st0 = 0, w0 = 0;  // the tile's first stage and weight slot
-    bool ok = true;
-    while (ok && walk.next()) {
-      const ColsTile& t = walk.t;
-      const int kb_n = t.up ? a.kb_up : a.kb_dn;
-      const uint32_t n_st = (kb_n + 3) / 4;
-      const int at = t.up ? at_up : at_dn;
-      const bool codes = t.g != g_sh;
-      // the stage that used this part of the TMEM ring (two before) has been consumed
-      auto stage_free = [&](uint32_t st) {
-        return st < 2 || wait_warp(&sempty[(st - 2) & s_mask], ((st - 2) >> s_log) & 1u, abort_flag, lim);
-      };
-      if (codes) {
-        // a slot is a stage: the set passes over one slot between its own
-        for (uint32_t i = (odd - st0) & 1u; i < n_st; i += 2) {
-          const uint32_t wc = w0 + i, wi = wc & w_mask;
-          if (!wait_warp(&wfull[wi], (wc >> w_log) & 1u, abort_flag, lim)) { ok = false; break; }
-          if (!stage_free(st0 + i)) { ok = false; break; }
-          if (4 * i + 2 * half < (uint32_t)kb_n) {
-            tc_fence_after();
-            // half a slot: 128 codes and four scales of the row
-            const uint32_t dst = tdst + set * 64;
-            const uint32_t src = sw0 + wi * kCSlot + at * 128 + ((half << 6) ^ x0);
-            const uint2 sc = ld_shared_v2(ss0 + wi * kCScale + at * 16 + half * 8);
-            const uint4 c0 = ld_shared_v4(src + x[0]), c1 = ld_shared_v4(src + x[1]);
-            convert32(c0, sc.x & 0xFFFFu, dst);
-            const uint4 c2 = ld_shared_v4(src + x[2]);
-            convert32(c1, sc.x >> 16, dst + 16);
-            const uint4 c3 = ld_shared_v4(src + x[3]);
-            convert32(c2, sc.y & 0xFFFFu, dst + 32);
-            convert32(c3, sc.y >> 16, dst + 48);
-            tmem_st_wait();
-            tc_fence_before();
-          }
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(&afull[set]);
-            mbar_arrive_n(&wempty[wi], 2);  // the warp's rows of the slot are consumed, for two sets
-          }
-        }
-      } else {
-        // 64 bf16 weights of each row a slot: every warp passes every slot
-        for (uint32_t kb = 0; kb < (uint32_t)kb_n; ++kb) {
-          const uint32_t st = st0 + (kb >> 2);
-          const uint32_t wc = w0 + kb, wi = wc & w_mask;
-          if (!wait_warp(&wfull[wi], (wc >> w_log) & 1u, abort_flag, lim)) { ok = false; break; }
-          if ((st & 1u) == odd && ((kb >> 1) & 1u) == half) {
-            if ((kb & 1u) == 0 && !stage_free(st)) { ok = false; break; }
-            tc_fence_after();
+    op.x0 = (lane & 4) << 4;
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-              const uint32_t src = sw0 + wi * kCSlot + at * 128 + ((p << 6) ^ x0);
-              const uint4 b0 = ld_shared_v4(src + x[0]), b1 = ld_shared_v4(src + x[1]);
-              const uint4 b2 = ld_shared_v4(src + x[2]), b3 = ld_shared_v4(src + x[3]);
-              const uint32_t o[16] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w,
-                                      b2.x, b2.y, b2.z, b2.w, b3.x, b3.y, b3.z, b3.w};
-              tmem_st16(tdst + set * 64 + (kb & 1u) * 32 + 16 * p, o);
-            }
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0 && (kb & 1u)) mbar_arrive(&afull[set]);
-          }
-          if (lane == 0) mbar_arrive(&wempty[wi]);
-        }
-        if (!ok) break;
-        if ((kb_n & 3) != 0 && half == 1 && ((st0 + n_st - 1) & 1u) == odd) {  // the last stage's missing half
-          if (!stage_free(st0 + n_st - 1)) break;
-          if (lane == 0) mbar_arrive(&afull[set]);
-        }
-      }
-      st0 += n_st;
-      w0 += codes ? n_st : kb_n;
+    for (int c = 0; c < 4; ++c) op.x[c] = ((uint32_t)c ^ (lane & 3u)) << 4;
+    while (walk.next()) {
+      const ColsTile& t = walk.t;
+      op.at = t.up ? at_up : at_dn;
+      if (!conv.tile(t.g != g_sh, t.up ? a.kb_up : a.kb_dn, op)) break;
     }
   }
 

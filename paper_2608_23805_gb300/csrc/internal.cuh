@@ -395,6 +395,77 @@ struct ColsWalk {
   }
 };
 
+// What a 4-bit conversion warp of gemm_cols.cu waits for, tile by tile, and in
+// which order.  Slots of the code ring and stages of the operand ring are
+// counted over the CTA's whole sequence.  Set j of the four sets of warps takes
+// half j & 1 of the stages of parity j >> 1: in a tile of codes a slot is a
+// stage, and a warp passes over every other slot; in a tile of the shared
+// expert four slots of 64 bf16 weights make a stage, and every warp waits for
+// every slot.
+//
+// A wait names its phase by a parity, so it holds only where the phase before
+// is known to be over: a slot that still waits for the load before the one that
+// is meant reads as if that one had landed.
+//  - Tile of codes after such: the slot's previous use was the warp's own.
+//  - Shared tile after a tile of codes (`unseen`): the slots' previous uses may
+//    have been the other parity's.  The warp waits until stage st0 - 1 has been
+//    consumed: MMAs complete in order, so every earlier slot has been filled and
+//    converted.  That wait in turn needs the same barrier's previous phase,
+//    stage st0 - 1 - ring: the warps of st0 - 1's parity have seen stage st0 - 3
+//    consumed, the others wait for st0 - 2 first.  Neither barrier can move on
+//    to its next phase meanwhile: the stage that ends it waits for this warp.
+//    The warps of st0 - 1's parity must not wait for st0 - 2: stage st0 may be
+//    consumed without them, which with two stages is that barrier's next phase.
+//  - After a shared tile the warp has seen its slots land, and knows the ones
+//    before it filled.
+struct ColsConvert {
+  uint32_t odd, half;        // of stages st with (st & 1) == odd, this half
+  uint32_t st0 = 0, w0 = 0;  // the tile's first stage and slot
+  bool unseen = false;
+
+  __host__ __device__ __forceinline__ explicit ColsConvert(uint32_t set) : odd(set >> 1), half(set & 1u) {}
+
+  // Op: slot(w): slot w's load has landed; stage(st): st's part of the operand
+  // ring is free (stage st - 2 consumed); codes(w, any): the half of slot w, if
+  // the tile's K reaches it, and its arrivals; rows(w, j): step j of the half
+  // from slot w, arriving with the second; none(): the half is empty; pass(w):
+  // done with slot w.  The waits return false when the launch aborts.
+#pragma nv_exec_check_disable
+  template <typename Op>
+  __host__ __device__ __forceinline__ bool tile(bool is_codes, uint32_t kb_n, Op& op) {
+    const uint32_t n_st = (kb_n + 3) / 4;
+    if (is_codes) {
+      for (uint32_t i = (odd - st0) & 1u; i < n_st; i += 2) {
+        if (!op.slot(w0 + i) || !op.stage(st0 + i)) return false;
+        op.codes(w0 + i, 4 * i + 2 * half < kb_n);
+      }
+      w0 += n_st;
+    } else {
+      if (unseen) {
+        if ((st0 & 1u) == odd && !op.stage(st0)) return false;
+        if (!op.stage(st0 + 1)) return false;
+      }
+      for (uint32_t kb = 0; kb < kb_n; ++kb) {
+        const uint32_t st = st0 + (kb >> 2);
+        if (!op.slot(w0 + kb)) return false;
+        if ((st & 1u) == odd && ((kb >> 1) & 1u) == half) {
+          if ((kb & 1u) == 0 && !op.stage(st)) return false;
+          op.rows(w0 + kb, kb & 1u);
+        }
+        op.pass(w0 + kb);
+      }
+      if ((kb_n & 3u) != 0 && half == 1 && ((st0 + n_st - 1) & 1u) == odd) {
+        if (!op.stage(st0 + n_st - 1)) return false;
+        op.none();
+      }
+      w0 += kb_n;
+    }
+    unseen = is_codes;
+    st0 += n_st;
+    return true;
+  }
+};
+
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
