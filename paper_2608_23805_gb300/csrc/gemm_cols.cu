@@ -305,8 +305,8 @@ __device__ __forceinline__ int cols_group_table(const FusedArgs& a, const W& w, 
     if (i < n) {
       if constexpr (wave) {
         e = w.expert[i];
-        cnt = __ldg(&a.counts[e]);
-        rb = __ldg(&a.offsets[e]);
+        cnt = a.counts[e];
+        rb = a.offsets[e];
         slot = w.slot[i];
         if (cnt > 0) {
           if (slot < 0) {
@@ -755,13 +755,13 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
       const int* perm = a.perm + s_rb[t.g] + row0;
       if (GATHER) {
         const int rr = min(4 * tw + 16 * (lane >> 2) + (lane & 3), rows - 1);
-        tok[0] = t.g == g_sh ? row0 + rr : __ldg(&perm[rr]);
+        tok[0] = t.g == g_sh ? row0 + rr : perm[rr];
       } else {
 #pragma unroll
         for (int i = 0; i < kRows; ++i) {
           if (16 * i >= rows) break;
           const int rr = r0 + 16 * i;
-          tok[i] = t.g == g_sh ? row0 + rr : rr < rows ? __ldg(&perm[rr]) : 0;
+          tok[i] = t.g == g_sh ? row0 + rr : rr < rows ? perm[rr] : 0;
         }
       }
     };

@@ -639,7 +639,9 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
 // while its predecessor in the stream still runs, and must not touch global
 // memory before grid_wait, which returns when the predecessor has completed and
 // its writes are visible.  Every kernel of such a chain waits, so each follows
-// all before it.  grid_release lets the successor start.
+// all before it.  What the chain writes is read by coherent loads (no __ldg:
+// the data change while the kernel is resident).  grid_release lets the
+// successor start.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

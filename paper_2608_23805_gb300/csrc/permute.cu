@@ -360,6 +360,12 @@ __device__ __forceinline__ void fma8(float (&acc)[8], float w, const uint4& y) {
   acc[7] = fmaf(w, bf16_hi(y.w), acc[7]);
 }
 
+// 16 bytes of a row the preceding kernels wrote.  A coherent load: the combine
+// is resident while they still run (launch_after).
+__device__ __forceinline__ uint4 row16(const __nv_bfloat16* rows, int r, int H, int c) {
+  return reinterpret_cast<const uint4*>(rows + (size_t)r * H)[c];
+}
+
 // One block per token; the token's k row indices and weights are read once
 // into shared memory, and up to eight expert rows are loaded before they are
 // summed (still in j order, fp32), so each thread keeps eight 16-byte loads
@@ -373,8 +379,8 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs a) {
   // rows' indices are a bijection in any case, and the load need not come first
   const int status = *a.status;
   if (threadIdx.x < a.k) {
-    s_row[threadIdx.x] = __ldg(&a.inv[(size_t)t * a.k + threadIdx.x]);
-    s_w[threadIdx.x] = __ldg(&a.weights[(size_t)t * a.k + threadIdx.x]);
+    s_row[threadIdx.x] = a.inv[(size_t)t * a.k + threadIdx.x];
+    s_w[threadIdx.x] = a.weights[(size_t)t * a.k + threadIdx.x];
   }
   __syncthreads();
   const int nchunk = a.H >> 3;
@@ -387,7 +393,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs a) {
       uint4 y[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u)
-        y[u] = __ldg(reinterpret_cast<const uint4*>(a.yp + (size_t)s_row[j + u] * a.H) + c);
+        y[u] = row16(a.yp, s_row[j + u], a.H, c);
 #pragma unroll
       for (int u = 0; u < 8; ++u) fma8(acc, s_w[j + u], y[u]);
     }
@@ -395,16 +401,15 @@ __global__ void __launch_bounds__(256) combine_kernel(const CombineArgs a) {
       uint4 y[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        y[u] = __ldg(reinterpret_cast<const uint4*>(a.yp + (size_t)s_row[j + u] * a.H) + c);
+        y[u] = row16(a.yp, s_row[j + u], a.H, c);
 #pragma unroll
       for (int u = 0; u < 4; ++u) fma8(acc, s_w[j + u], y[u]);
       j += 4;
     }
     for (; j < a.k; ++j)
-      fma8(acc, s_w[j], __ldg(reinterpret_cast<const uint4*>(a.yp + (size_t)s_row[j] * a.H) + c));
+      fma8(acc, s_w[j], row16(a.yp, s_row[j], a.H, c));
     if (a.ys != nullptr)  // gate sigmoid(x . w_sg), or 1 for an ungated shared expert
-      fma8(acc, a.sg != nullptr ? a.sg[t] : 1.0f,
-           __ldg(reinterpret_cast<const uint4*>(a.ys + (size_t)t * a.H) + c));
+      fma8(acc, a.sg != nullptr ? a.sg[t] : 1.0f, row16(a.ys, t, a.H, c));
     if (a.x != nullptr) {
       const uint4 y = __ldg(reinterpret_cast<const uint4*>(a.x + (size_t)t * a.H) + c);
       acc[0] += bf16_lo(y.x);
