@@ -389,9 +389,12 @@ WsLayout layout(const msi_plan* p, int T) {
   L.h = take(2 * Tk * I);
   L.yp = take(2 * Tk * H);
   // fused GEMMs: a counter per 128-row tile, two banks (consecutive waves
-  // alternate; each wave's kernel zeroes the other bank for the next)
-  const size_t tile = cols_tile_tokens((long long)Tk, (int)E);
-  L.ready_n = Tk / tile + E + 1 + (p->d.has_shared ? (size_t)T / tile + 1 : 0);
+  // alternate; each wave's kernel zeroes the other bank for the next).  The
+  // smaller token tiles of gemm_cols.cu fit too: a resident call counts across
+  // both banks (32-token tiles up to 10 rows a group, 64 up to 24: with the
+  // shared expert's, (Tk + T) / tile + E + 2 <= 2 (Tk / 128 + E + 1)), a wave
+  // takes larger tiles where its bank is too small (routed_ffn)
+  L.ready_n = Tk / kBM + E + 1;
   L.ready = take(2 * 4 * L.ready_n);
   if (p->d.has_shared) {
     L.hs = take(2 * (size_t)T * I);
@@ -949,7 +952,7 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
     xa.layer = tp.layer;
     if (fused_resident(p, f, (long long)f.T * k, E) || cols) {
       xa.ready = at<int>(ws, L.ready);
-      xa.n_ready = ready_bank(f);
+      xa.n_ready = (cols ? 2 : 1) * ready_bank(f);
     }
   } else if (!(f.flags & MSI_FWD_SPLIT_WAVES)) {
     // streamed call: the first fused wave's bank (later waves' banks are
@@ -1113,6 +1116,7 @@ msi_status routed_ffn(msi_plan* p, FwdCtx& f, int ng, int grid1, int grid2, long
     }
     if (cols) {
       fa.tile_tok = std::max(cols_tile_tokens(rows, ng), cols_tile_tokens((long long)f.T * d.top_k, d.n_experts));
+      while (wp != nullptr && fa.tile_tok < kBM && rows / fa.tile_tok + ng > (long long)f.L.ready_n) fa.tile_tok *= 2;
       fa.nt_up = d.inter / 64;
       fa.nt_dn = d.hidden / 128;
       long long all = (long long)wave_mtiles * (fa.nt_up + fa.nt_dn);

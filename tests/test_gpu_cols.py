@@ -15,9 +15,9 @@ from gpu_case import Case, bf16_bits, bf16_tensor, compare_out, compare_routes
 pytestmark = pytest.mark.gpu
 
 
-def run_case(tokens, wdtype, streamed, hidden, inter, experts, top_k, shared, residual=False):
+def run_case(tokens, wdtype, streamed, hidden, inter, experts, top_k, shared, residual=False, slots=8):
     cfg = synth.config("tiny", hidden=hidden, inter=inter, n_experts=experts, top_k=top_k, tokens=tokens,
-                       n_slots=8 if streamed else experts, wdtype=wdtype, has_shared=shared)
+                       n_slots=slots if streamed else experts, wdtype=wdtype, has_shared=shared)
     case = Case(cfg)
     x_bits = synth.hidden(cfg)
     x = bf16_tensor(x_bits)
@@ -52,6 +52,13 @@ def test_q4_lengths(tokens, streamed):
 @pytest.mark.parametrize("shared", [False, True])
 def test_q4_shapes(hidden, inter, experts, top_k, shared):
     run_case(90, synth.W_Q4G32, False, hidden, inter, experts, top_k, shared, residual=True)
+
+
+@pytest.mark.parametrize("tokens", [70, 80])
+def test_q4_wave_of_all_groups(tokens):
+    # one wave of all 32 groups of ~10 rows: more 32-token tiles than a bank
+    # of counters may hold
+    run_case(tokens, synth.W_Q4G32, True, 512, 256, 32, 4, False, slots=64)
 
 
 @pytest.mark.parametrize("tokens", [1, 3, 16, 17, 40])

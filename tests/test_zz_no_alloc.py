@@ -97,3 +97,16 @@ def test_static_scratch_limit_at_qwen_shape():
     # a call after the rejection is still exact
     _check_equal(case, table, gens, 100, 1)
     case.close()
+
+
+@pytest.mark.parametrize("hidden,inter,experts,top_k,limit", [(256, 256, 16, 2, 10834), (1792, 640, 16, 8, 765)])
+def test_static_scratch_limit_at_small_shapes(hidden, inter, experts, top_k, limit):
+    """Layers with a shared expert whose longest call leaves less room in the
+    array than a few counters take."""
+    cfg = synth.config("tiny", hidden=hidden, inter=inter, n_experts=experts, top_k=top_k, n_slots=experts,
+                       tokens=limit, has_shared=True)
+    case = Case(cfg)
+    table, gens = case.stage_all()
+    assert _ws_bytes(case.plan, limit) <= STATIC_SCRATCH_BYTES < _ws_bytes(case.plan, limit + 1)
+    _check_equal(case, table, gens, limit, 0)
+    case.close()
