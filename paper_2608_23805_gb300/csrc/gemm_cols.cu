@@ -13,7 +13,8 @@
 //       gate, ... (lanes 16 apart hold gate and up of a unit, one shuffle
 //       brings them together): h[rows, 64 n .. 64 n + 64) = silu(g) * u
 //   down tile (g, m, n):  128 output features: y[rows, 128 n .. 128 n + 128)
-// The resident shared expert is one more group (all tokens, identity rows).
+// A short resident call's shared expert is one more group (all tokens, identity
+// rows; cols_shared in plan.cu).
 //
 // K goes by stages of four steps of 64 (two where four would leave too few
 // stages), one tcgen05.commit a stage: the issuing and the token warp's

@@ -740,24 +740,43 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
   return MSI_OK;
 }
 
-// Weights as MMA rows (gemm_cols.cu), in one launch with a resident call's
-// shared expert, while the groups average few rows:
+// Weights as MMA rows (gemm_cols.cu) while the groups average few rows:
 //   4-bit: at 8, 250 and 4,096 tokens of the Qwen-shaped layer 62, 288 and 416
 //     us against 91, 534 and 546 in two row-major launches; the call at 8,192
 //     tokens 964 against 1,209, at 20,000 (390 rows a group, four tiles and
 //     conversions) 2,105 against 2,215, at 32,768 3,508 against 3,086 on pairs.
 //     A wave up to 256 rows.
-//   bf16: where the launches' latency is what counts (one token: 24 us for
-//     what took 28 + 25 on a side stream).  From some 40 tokens on both
-//     orientations stream the weights at the same rate (0.97 of HBM), and the
-//     row-major tiles read the tokens half as often (the call at 300 tokens 532
-//     in both, at 600 541 row-major and 543 here, at 2,000 581 and 607).  Not a wave: its launch has no
-//     shared expert to take in.
+//   bf16: where the launches' latency is what counts, up to 256 rows with a
+//     shared expert, which this launch takes in (one token: 24 us for what took
+//     28 + 25 on a side stream).  Calls, us, row-major and here, top_k 10 of 512
+//     experts: 37 rows 294 and 290, 200 rows 513 and 513, 400 rows 532 and 538;
+//     top_k 1 of 256: 250 rows 198 and 196, 1,000 rows 297 and 310, 2,000 rows
+//     310 and 343; top_k 1 of 16, 120 rows: 113 and 96.  Both orientations
+//     stream the weights at the same rate (0.97 of HBM), and the row-major
+//     tiles read the tokens half as often.  Without a shared expert only while
+//     the up tiles are one round of the SMs (top_k 1 of 16, 100 rows: 94 and
+//     90; top_k 2 of 64, 100 rows, 3.4 rounds: 98 and 108).  Not a wave: its
+//     launch has no shared expert to take in.
 constexpr long long kColsMaxRows = 512, kColsMaxRowsWave = 256, kColsMaxRowsBf16 = 8;
+constexpr int kColsMaxCallBf16 = 256;
 bool cols_tiles(const msi_plan* p, const FwdCtx& f, long long rows, int ng, bool wave = false) {
-  return !(f.flags & (MSI_FWD_SPLIT_WAVES | MSI_FWD_SINGLE_CTA)) && ng > 0 &&
-         rows < (wave ? kColsMaxRowsWave : kColsMaxRows) * ng &&
-         (p->d.wdtype == MSI_W_Q4G32 || (!wave && rows < kColsMaxRowsBf16 * ng));
+  if ((f.flags & (MSI_FWD_SPLIT_WAVES | MSI_FWD_SINGLE_CTA)) || ng < 1 ||
+      rows >= (wave ? kColsMaxRowsWave : kColsMaxRows) * ng)
+    return false;
+  if (p->d.wdtype == MSI_W_Q4G32) return true;
+  if (wave || rows >= kColsMaxRowsBf16 * ng) return false;
+  return p->d.has_shared ? f.T <= kColsMaxCallBf16 : std::min<long long>(rows, ng) * (p->d.inter / 64) <= p->sms;
+}
+
+// Such a resident call's shared expert: in its launch, or from 65 rows of a
+// 4-bit layer, where its bf16 weights pass through the conversion warps once a
+// tile, in launches of its own on the side stream (us, in the launch and
+// beside it: top_k 10 of 512 experts, 8 rows 100 and 107, 64 rows 246 and 249,
+// 128 rows 304 and 300, 4,096 rows 535 and 508; top_k 2 of 64, 64 rows 93 and
+// 95, 200 rows 107 and 102; top_k 1 of 256, 2,000 rows 260 and 214).
+constexpr int kColsMaxSharedQ4 = 64;
+bool cols_shared(const msi_plan* p, const FwdCtx& f) {
+  return p->d.has_shared && (p->d.wdtype == MSI_W_BF16 || f.T <= kColsMaxSharedQ4);
 }
 
 // Router + histogram over the call's rows for router weight `rw`: the route
@@ -820,7 +839,8 @@ msi_status route_rows(msi_plan* p, FwdCtx& f, const float* rw, const msi_route_e
     const bool fuse = first && xa != nullptr && f.T <= kFuseTokens;
     // a long resident call begins with a kernel of its own, so that the side
     // stream's shared expert runs beside the logits and not after them
-    const bool begun = first && tp.E > 0 && d.has_shared && f.T >= 4096 && !cols_tiles(p, f, (long long)f.T * k, E);
+    const bool begun = first && tp.E > 0 && d.has_shared && f.T >= 4096 &&
+                       !(cols_tiles(p, f, (long long)f.T * k, E) && cols_shared(p, f));
     if (begun) {
       LAUNCH(p, MSI_K_UPLOAD, s, launch_upload(tp, ra.tab_slot, ra.tab_expected, ra.status, ra.sh, ra.sh_total, s));
       CK(cudaEventRecord(p->ev_fork, s));
@@ -916,7 +936,7 @@ msi_status front(msi_plan* p, FwdCtx& f, const TableParams& tp) {
   const int nb = (f.T + L.tm - 1) / L.tm;
   if (!make_tmap(&f.tm_x, f.x, H, f.T, 128)) return MSI_ERR_CUDA;
   const bool cols = tp.E > 0 && cols_tiles(p, f, (long long)f.T * k, E);  // the row-major kernels' maps are not needed
-  if (d.has_shared && !cols) {
+  if (d.has_shared && !(cols && cols_shared(p, f))) {
     if (!make_tmap(&f.tm_hs, at<char>(ws, L.hs), I, f.T, 128)) return MSI_ERR_CUDA;
   }
   // up to kScatterWarps router blocks: one scatter block covers them all and
@@ -1120,7 +1140,7 @@ msi_status routed_ffn(msi_plan* p, FwdCtx& f, int ng, int grid1, int grid2, long
       fa.nt_up = d.inter / 64;
       fa.nt_dn = d.hidden / 128;
       long long all = (long long)wave_mtiles * (fa.nt_up + fa.nt_dn);
-      if (wp == nullptr && d.has_shared) {
+      if (wp == nullptr && cols_shared(p, f)) {
         fa.sh_rows = f.T;
         fa.sh_slot = f.layer;
         fa.hs = at<__nv_bfloat16>(f.ws, f.L.hs);
@@ -1576,7 +1596,7 @@ msi_status forward_resident(msi_plan* p, int layer, const void* x, int T, const 
   st = front(p, f, tp);
   if (st != MSI_OK) return st;
   const bool cols = cols_tiles(p, f, (long long)T * d.top_k, E);
-  const bool fork = d.has_shared && T > 0 && !cols;
+  const bool fork = d.has_shared && T > 0 && !(cols && cols_shared(p, f));
   if (fork) {
     // the shared expert needs no routing: it runs on the side stream while
     // the router, scan and scatter leave most SMs idle, and joins before the

@@ -70,3 +70,35 @@ def test_bf16_lengths(tokens, streamed):
 @pytest.mark.parametrize("hidden,inter,experts,top_k", [(256, 128, 16, 2), (768, 384, 32, 1), (1024, 640, 64, 8)])
 def test_bf16_shapes(hidden, inter, experts, top_k):
     run_case(20, synth.W_BF16, False, hidden, inter, experts, top_k, True)
+
+
+@pytest.mark.parametrize("wdtype,hidden,experts,top_k,tokens,launches", [
+    # the shared expert in the FFN's launch up to 64 rows of a 4-bit layer,
+    # else in two of its own
+    (synth.W_Q4G32, 512, 16, 2, 64, (1, 0, 0)), (synth.W_Q4G32, 512, 16, 2, 65, (1, 1, 0)),
+    # a bf16 layer: in the FFN's launch on weights as rows (to 256 rows, 8 a
+    # group), else beside the row-major one
+    (synth.W_BF16, 256, 64, 1, 256, (1, 0, 0)), (synth.W_BF16, 256, 64, 1, 257, (1, 1, 0)),
+    (synth.W_BF16, 256, 16, 4, 32, (1, 1, 0)),
+    # 512 rows a group: two row-major launches
+    (synth.W_Q4G32, 256, 4, 1, 2048, (0, 1, 1))])
+def test_routes(wdtype, hidden, experts, top_k, tokens, launches):
+    cfg = synth.config("tiny", hidden=hidden, inter=128, n_experts=experts, top_k=top_k, tokens=tokens,
+                       n_slots=experts, wdtype=wdtype, has_shared=True)
+    case = Case(cfg)
+    table, gens = case.stage_all()
+    x_bits = synth.hidden(cfg)
+    case.plan.timing(True)
+    out, _ = case.plan.forward(0, bf16_tensor(x_bits), case.router[0], table, gens)
+    torch.cuda.synchronize()
+    n = {k: v[1] for k, v in case.plan.timing_read().items()}
+    assert (n["ffn"], n["shared_gateup"], n["gateup"]) == launches
+    compare_out(bf16_bits(out), case.oracle_layer(x_bits)["out"])
+    case.close()
+
+
+@pytest.mark.parametrize("hidden,inter", [(256, 128), (768, 128), (1280, 640)])
+def test_q4_shared_expert_in_large_tiles(hidden, inter):
+    # 128-token tiles, and shared and routed tiles of an odd and an even number
+    # of weight slots and stages
+    run_case(60, synth.W_Q4G32, False, hidden, inter, 16, 8, True)
