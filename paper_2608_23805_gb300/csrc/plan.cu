@@ -837,20 +837,16 @@ msi_status route_rows(msi_plan* p, FwdCtx& f, const float* rw, const msi_route_e
     ra.chunk = router_chunk(chunk_rows, E, p->sms);
     ra.nchunk = E / ra.chunk;
     const bool fuse = first && xa != nullptr && f.T <= kFuseTokens;
-    // a long resident call begins with a kernel of its own, so that the side
-    // stream's shared expert runs beside the logits and not after them
-    const bool begun = first && tp.E > 0 && d.has_shared && f.T >= 4096 &&
-                       !(cols_tiles(p, f, (long long)f.T * k, E) && cols_shared(p, f));
-    if (begun) {
-      LAUNCH(p, MSI_K_UPLOAD, s, launch_upload(tp, ra.tab_slot, ra.tab_expected, ra.status, ra.sh, ra.sh_total, s));
-      CK(cudaEventRecord(p->ev_fork, s));
-    }
     for (ra.t0 = 0; ra.t0 < f.T; ra.t0 += chunk_rows) {
       ra.rows = std::min(chunk_rows, f.T - ra.t0);
-      ra.begin = first && !begun && ra.t0 == 0;
+      ra.begin = first && ra.t0 == 0;
       LAUNCH(p, MSI_K_ROUTER, s, launch_router_logits(f.tm_x, ra, tp, s));
       // the forward has begun (status cleared, shared group written): the
-      // shared expert may start on the side stream from here
+      // shared expert may start on the side stream from here.  Beside the
+      // logits, after a kernel of its own that begins the call, it delays them
+      // by as much or more (us, so and here: bf16 4,096 rows 644 and 645,
+      // 16,000 rows 1,325 and 1,311; 4-bit 4,096 rows 507 and 508, 8,192 rows
+      // 940 and 912; 64 experts, H 1,024, 8,000 rows 133 and 124)
       if (ra.begin && d.has_shared) CK(cudaEventRecord(p->ev_fork, s));
       LAUNCH(p, MSI_K_ROUTER, s, launch_router_select(ra, fuse ? xa : nullptr, s));
     }
