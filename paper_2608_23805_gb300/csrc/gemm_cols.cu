@@ -855,7 +855,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
         }
         const uint32_t dst0 = smem_u32(sT) + w_stage + r0 * 128 + ((chunk ^ (r0 & 7)) << 4);
         for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-          if (!mbar_wait(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+          if (!wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
           const uint32_t dst = dst0 + r.i * stage;
 #pragma unroll
           for (int i = 0; i < kRows; ++i) {

@@ -92,7 +92,7 @@ __device__ __forceinline__ void split_weights(const float* src, int H, int nstag
   if (group < nstage) load(group);
   for (int it = group; it < nstage; it += C::kGroups) {
     const int s = it % C::kStages;
-    if (!mbar_wait(&empty[s], ((it / C::kStages) & 1) ^ 1, abort_flag, lim)) return;
+    if (!mbar_wait_warp(&empty[s], ((it / C::kStages) & 1) ^ 1, abort_flag, lim)) return;
     const uint32_t st = smem_u32(smem + s * C::kStage) + kXBytes;
 #pragma unroll
     for (int i = 0; i < C::kVec; ++i) {
