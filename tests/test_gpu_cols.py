@@ -11,6 +11,7 @@ import torch
 
 import synth
 from gpu_case import Case, bf16_bits, bf16_tensor, compare_out, compare_routes
+from paper_2608_23805_gb300 import native as N
 
 pytestmark = pytest.mark.gpu
 
@@ -62,9 +63,14 @@ def test_q4_wave_of_all_groups(tokens):
 
 
 @pytest.mark.parametrize("tokens", [1, 3, 16, 17, 40])
-@pytest.mark.parametrize("streamed", [False, True])
-def test_bf16_lengths(tokens, streamed):
-    run_case(tokens, synth.W_BF16, streamed, 512, 256, 64, 8, not streamed)
+def test_bf16_lengths(tokens):
+    run_case(tokens, synth.W_BF16, False, 512, 256, 64, 8, True)
+
+
+@pytest.mark.parametrize("tokens", [1, 9, 60])
+def test_bf16_without_shared_expert(tokens):
+    # the kernel's while min(rows, experts) I / 64 fits the SMs
+    run_case(tokens, synth.W_BF16, False, 512, 256, 32, 2, False)
 
 
 @pytest.mark.parametrize("hidden,inter,experts,top_k", [(256, 128, 16, 2), (768, 384, 32, 1), (1024, 640, 64, 8)])
@@ -102,3 +108,92 @@ def test_q4_shared_expert_in_large_tiles(hidden, inter):
     # 128-token tiles, and shared and routed tiles of an odd and an even number
     # of weight slots and stages
     run_case(60, synth.W_Q4G32, False, hidden, inter, 16, 8, True)
+
+
+# calls on this kernel with each of its token paths and groups: the shared
+# expert inside, 128-token tiles, a wave, bf16 behind the tensor router, bf16
+FORMS = [(synth.W_Q4G32, False, 512, 256, 16, 4, 40, True), (synth.W_Q4G32, False, 512, 256, 16, 4, 700, True),
+         (synth.W_Q4G32, True, 512, 256, 16, 4, 90, False), (synth.W_BF16, False, 1024, 256, 64, 4, 50, True),
+         (synth.W_BF16, False, 256, 128, 64, 1, 200, True)]
+
+
+def form_case(wdtype, streamed, hidden, inter, experts, top_k, tokens, shared):
+    cfg = synth.config("tiny", hidden=hidden, inter=inter, n_experts=experts, top_k=top_k, tokens=tokens,
+                       n_slots=8 if streamed else experts, wdtype=wdtype, has_shared=shared)
+    case = Case(cfg)
+    table = None if streamed else case.stage_all()
+
+    def call(x, out):
+        if streamed:
+            return case.plan.forward_streamed(0, x, case.router[0], out=out)
+        return case.plan.forward(0, x, case.router[0], *table, out=out)
+
+    return cfg, case, call
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_expired_wait_fails_closed_then_recovers(form):
+    # one wait of each launch that nothing ends, with a limit of ~1 ms: the
+    # launch gives up, lands its copies and reports a timeout
+    cfg, case, call = form_case(*form)
+    x_bits = synth.hidden(cfg)
+    x = bf16_tensor(x_bits)
+    out = torch.full_like(x, 7.0)
+    case.plan.set_wait_cycles(2_000_000)
+    case.plan.inject(N.MSI_FAULT_DEVICE_WAIT, 0, 0)
+    call(x, out)
+    torch.cuda.synchronize()
+    assert case.plan.status() == N.MSI_ERR_TIMEOUT
+    assert torch.all(out == 7.0)
+    case.plan.set_wait_cycles(0)
+    call(x, out)
+    torch.cuda.synchronize()
+    assert case.plan.status() == N.MSI_OK
+    compare_out(bf16_bits(out), case.oracle_layer(x_bits)["out"])
+    case.close()
+
+
+@pytest.mark.parametrize("kind,status", [(N.MSI_FAULT_STALE_COMPLETION, N.MSI_ERR_STALE_GENERATION),
+                                         (N.MSI_FAULT_WRONG_OBJECT, N.MSI_ERR_WRONG_OBJECT)])
+@pytest.mark.parametrize("form", [FORMS[0], FORMS[2]])
+def test_wrong_publication_fails_closed(form, kind, status):
+    # a slot whose published word is not the plan's: the launch (a wave), or the
+    # scatter before it, rejects its group and no row becomes visible
+    streamed = form[1]
+    cfg, case, call = form_case(*form)
+    x_bits = synth.hidden(cfg)
+    x = bf16_tensor(x_bits)
+    used = np.unique(case.oracle_layer(x_bits)["ids"])
+    out = torch.full_like(x, 5.0)
+    e = int(used[len(used) // 2])
+    case.plan.inject(kind, 0, e)
+    if not streamed:
+        case.plan.stage(e, 0, e)
+        gens = case.plan.slot_table(0)
+        case.plan.forward(0, x, case.router[0], *gens, out=out)
+    else:
+        call(x, out)
+    torch.cuda.synchronize()
+    assert case.plan.status() == status
+    assert torch.all(out == 5.0)
+    case.close()
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_back_to_back_calls_on_one_workspace(form):
+    # four chained calls with other inputs, nothing waited for between them:
+    # each output is that of the same call alone
+    cfg, case, call = form_case(*form)
+    xs = [bf16_tensor(synth.hidden(cfg, 0, i)) for i in range(4)]
+    outs = [torch.empty_like(x) for x in xs]
+    for x, out in zip(xs, outs):
+        call(x, out)
+    torch.cuda.synchronize()
+    assert case.plan.status() == N.MSI_OK
+    for x, out in zip(xs, outs):
+        alone = torch.empty_like(x)
+        call(x, alone)
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int16), alone.view(torch.int16))
+    compare_out(bf16_bits(outs[3]), case.oracle_layer(synth.hidden(cfg, 0, 3))["out"])
+    case.close()
