@@ -745,7 +745,14 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 //     us against 91, 534 and 546 in two row-major launches; the call at 8,192
 //     tokens 964 against 1,209, at 20,000 (390 rows a group, four tiles and
 //     conversions) 2,105 against 2,215, at 32,768 3,508 against 3,086 on pairs.
-//     A wave up to 256 rows.
+//     64 experts, H 1,024, I 512, top_k 2: 4,000 to 14,000 rows 111 to 233
+//     against 120 to 244.  Small experts (few K steps and little to convert a
+//     tile, so that its hand-overs count) up to 24 rows a group: the call at 8,
+//     22, 47, 62 and 125 rows a group (H 512, I 256) 55, 66, 70, 75 and 92
+//     against 60, 69, 70, 70 and 88; H 2,048, I 128 at 31 rows 116 against 100;
+//     H 256, I 768 at 16 and 31 rows 111 and 126 against 118 and 119.
+//     A wave up to 256 rows (streamed calls of small experts, H 512, I 256: 16,
+//     62 and 125 rows a group 173, 200 and 209 against 208, 215 and 223).
 //   bf16: where the launches' latency is what counts, up to 256 rows with a
 //     shared expert, which this launch takes in (one token: 24 us for what took
 //     28 + 25 on a side stream).  Calls, us, row-major and here, top_k 10 of 512
@@ -758,10 +765,12 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 //     90; top_k 2 of 64, 100 rows, 3.4 rounds: 98 and 108).  Not a wave: its
 //     launch has no shared expert to take in.
 constexpr long long kColsMaxRows = 512, kColsMaxRowsWave = 256, kColsMaxRowsBf16 = 8;
+constexpr long long kColsMaxRowsSmall = 24;
 constexpr int kColsMaxCallBf16 = 256;
+bool small_experts(const msi_plan_desc& d) { return d.inter < 256 || (long long)d.hidden * d.inter < 262144; }
 bool cols_tiles(const msi_plan* p, const FwdCtx& f, long long rows, int ng, bool wave = false) {
   if ((f.flags & (MSI_FWD_SPLIT_WAVES | MSI_FWD_SINGLE_CTA)) || ng < 1 ||
-      rows >= (wave ? kColsMaxRowsWave : kColsMaxRows) * ng)
+      rows >= (wave ? kColsMaxRowsWave : small_experts(p->d) ? kColsMaxRowsSmall : kColsMaxRows) * ng)
     return false;
   if (p->d.wdtype == MSI_W_Q4G32) return true;
   if (wave || rows >= kColsMaxRowsBf16 * ng) return false;

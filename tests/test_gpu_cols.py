@@ -45,7 +45,7 @@ def run_case(tokens, wdtype, streamed, hidden, inter, experts, top_k, shared, re
 @pytest.mark.parametrize("tokens", [1, 2, 15, 17, 33, 64, 129, 500, 700])
 @pytest.mark.parametrize("streamed", [False, True])
 def test_q4_lengths(tokens, streamed):
-    run_case(tokens, synth.W_Q4G32, streamed, 512, 256, 16, 4, not streamed)
+    run_case(tokens, synth.W_Q4G32, streamed, 512, 512, 16, 4, not streamed)
 
 
 @pytest.mark.parametrize("hidden,inter,experts,top_k", [(256, 128, 16, 2), (768, 384, 8, 1), (1024, 640, 24, 8),
@@ -78,18 +78,19 @@ def test_bf16_shapes(hidden, inter, experts, top_k):
     run_case(20, synth.W_BF16, False, hidden, inter, experts, top_k, True)
 
 
-@pytest.mark.parametrize("wdtype,hidden,experts,top_k,tokens,launches", [
+@pytest.mark.parametrize("wdtype,hidden,inter,experts,top_k,tokens,launches", [
     # the shared expert in the FFN's launch up to 64 rows of a 4-bit layer,
     # else in two of its own
-    (synth.W_Q4G32, 512, 16, 2, 64, (1, 0, 0)), (synth.W_Q4G32, 512, 16, 2, 65, (1, 1, 0)),
+    (synth.W_Q4G32, 512, 128, 16, 2, 64, (1, 0, 0)), (synth.W_Q4G32, 512, 128, 16, 2, 65, (1, 1, 0)),
+    # two row-major launches from 24 rows a group of small experts, from 512
+    (synth.W_Q4G32, 256, 128, 4, 1, 95, (1, 1, 0)), (synth.W_Q4G32, 256, 128, 4, 1, 96, (0, 1, 1)),
+    (synth.W_Q4G32, 512, 512, 4, 1, 2047, (1, 1, 0)), (synth.W_Q4G32, 512, 512, 4, 1, 2048, (0, 1, 1)),
     # a bf16 layer: in the FFN's launch on weights as rows (to 256 rows, 8 a
     # group), else beside the row-major one
-    (synth.W_BF16, 256, 64, 1, 256, (1, 0, 0)), (synth.W_BF16, 256, 64, 1, 257, (1, 1, 0)),
-    (synth.W_BF16, 256, 16, 4, 32, (1, 1, 0)),
-    # 512 rows a group: two row-major launches
-    (synth.W_Q4G32, 256, 4, 1, 2048, (0, 1, 1))])
-def test_routes(wdtype, hidden, experts, top_k, tokens, launches):
-    cfg = synth.config("tiny", hidden=hidden, inter=128, n_experts=experts, top_k=top_k, tokens=tokens,
+    (synth.W_BF16, 256, 128, 64, 1, 256, (1, 0, 0)), (synth.W_BF16, 256, 128, 64, 1, 257, (1, 1, 0)),
+    (synth.W_BF16, 256, 128, 16, 4, 32, (1, 1, 0))])
+def test_routes(wdtype, hidden, inter, experts, top_k, tokens, launches):
+    cfg = synth.config("tiny", hidden=hidden, inter=inter, n_experts=experts, top_k=top_k, tokens=tokens,
                        n_slots=experts, wdtype=wdtype, has_shared=True)
     case = Case(cfg)
     table, gens = case.stage_all()
@@ -103,16 +104,16 @@ def test_routes(wdtype, hidden, experts, top_k, tokens, launches):
     case.close()
 
 
-@pytest.mark.parametrize("hidden,inter", [(256, 128), (768, 128), (1280, 640)])
-def test_q4_shared_expert_in_large_tiles(hidden, inter):
-    # 128-token tiles, and shared and routed tiles of an odd and an even number
-    # of weight slots and stages
-    run_case(60, synth.W_Q4G32, False, hidden, inter, 16, 8, True)
+@pytest.mark.parametrize("hidden,inter,tokens", [(256, 128, 47), (768, 128, 47), (1280, 640, 60), (1024, 256, 60)])
+def test_q4_shared_expert_in_large_tiles(hidden, inter, tokens):
+    # 64- and 128-token tiles, and shared and routed tiles of an odd and an even
+    # number of weight slots and stages
+    run_case(tokens, synth.W_Q4G32, False, hidden, inter, 16, 8, True)
 
 
 # calls on this kernel with each of its token paths and groups: the shared
 # expert inside, 128-token tiles, a wave, bf16 behind the tensor router, bf16
-FORMS = [(synth.W_Q4G32, False, 512, 256, 16, 4, 40, True), (synth.W_Q4G32, False, 512, 256, 16, 4, 700, True),
+FORMS = [(synth.W_Q4G32, False, 512, 256, 16, 4, 40, True), (synth.W_Q4G32, False, 512, 512, 16, 4, 700, True),
          (synth.W_Q4G32, True, 512, 256, 16, 4, 90, False), (synth.W_BF16, False, 1024, 256, 64, 4, 50, True),
          (synth.W_BF16, False, 256, 128, 64, 1, 200, True)]
 
