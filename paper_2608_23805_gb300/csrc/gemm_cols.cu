@@ -72,18 +72,8 @@ constexpr int kCDqWarp0 = 10;
 constexpr int kCDqWarps = 16;
 constexpr int kCTable = kMaxExperts + 1;  // groups: experts and the shared one
 
-// GATHER: x by TMA gathers (tiles of up to 64 tokens)
-template <bool Q4, int STEPS, bool GATHER>
-struct CCfg {
-  static constexpr int kThreads = (kCDqWarp0 + (Q4 ? kCDqWarps : 0)) * 32;
-  static constexpr uint32_t kOperandCol = 256;  // TMEM: two accumulators of 128 columns, then A steps
-};
-
-// mbar_wait by a whole warp, which is converged after it (what follows may be
-// an aligned TMEM access), with one answer.
-__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit));
-}
+constexpr uint32_t kCOperandCol = 256;    // TMEM: two accumulators of 128 columns, then A steps
+constexpr int cols_threads(bool q4) { return (kCDqWarp0 + (q4 ? kCDqWarps : 0)) * 32; }
 
 // Ring position: slot index and the parity of its round.
 struct Ring {
@@ -216,10 +206,10 @@ struct ConvertOps {
   int lane, at;
 
   __device__ __forceinline__ bool slot(uint32_t w) const {
-    return wait_warp(&wfull[w & (a.ring_w - 1)], (w & a.ring_w) != 0, abort_flag, a.wait_limit);
+    return mbar_wait_warp(&wfull[w & (a.ring_w - 1)], (w & a.ring_w) != 0, abort_flag, a.wait_limit);
   }
   __device__ __forceinline__ bool stage(uint32_t st) const {
-    return st < 2 || wait_warp(&sempty[(st - 2) & (a.ring_s - 1)], ((st - 2) & a.ring_s) != 0, abort_flag, a.wait_limit);
+    return st < 2 || mbar_wait_warp(&sempty[(st - 2) & (a.ring_s - 1)], ((st - 2) & a.ring_s) != 0, abort_flag, a.wait_limit);
   }
   __device__ __forceinline__ void codes(uint32_t w, bool any) const {
     const uint32_t wi = w & (a.ring_w - 1);
@@ -375,14 +365,14 @@ __device__ __forceinline__ int cols_group_table(const FusedArgs& a, const W& w, 
 
 }  // namespace
 
+// GATHER: x by TMA gathers (tiles of up to 64 tokens)
 template <bool Q4, int STEPS, bool GATHER, typename W>
-__global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
+__global__ void __launch_bounds__(cols_threads(Q4), 1)
     fused_cols_kernel(const __grid_constant__ CUtensorMap tmW13, const __grid_constant__ CUtensorMap tmW2,
                       const __grid_constant__ CUtensorMap tmS13, const __grid_constant__ CUtensorMap tmS2,
                       const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmH,
                       const __grid_constant__ CUtensorMap tmHS, const __grid_constant__ FusedArgs a,
                       const __grid_constant__ W w) {
-  using C = CCfg<Q4, STEPS, GATHER>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -593,11 +583,11 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
       const int kb_n = (int)uniform(t.up ? a.kb_up : a.kb_dn);
       const uint32_t cols = uniform(min(a.tile_tok, s_cnt[t.g] - t.m * a.tile_tok));
       const uint32_t idesc = idesc_bf16(128, (cols + 15) & ~15);
-      ok = wait_warp(&tempty[acc], aph ^ 1, abort_flag, lim);
+      ok = mbar_wait_warp(&tempty[acc], aph ^ 1, abort_flag, lim);
       if (!ok) break;
       const uint32_t d = tm + acc * 128;
       for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-        ok = wait_warp(&sfull[r.i], r.ph, abort_flag, lim);
+        ok = mbar_wait_warp(&sfull[r.i], r.ph, abort_flag, lim);
         if (!ok) break;
         // cp.async (generic proxy) wrote the tokens: before the tensor core's reads
         if (!GATHER) fence_proxy_async_smem();
@@ -608,10 +598,10 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
           // past the tile's K has its second half announced empty)
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            ok = wait_warp(&afull[ra.i], ra.ph, abort_flag, lim);
+            ok = mbar_wait_warp(&afull[ra.i], ra.ph, abort_flag, lim);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t at = tm + C::kOperandCol + ra.i * 64;
+            const uint32_t at = tm + kCOperandCol + ra.i * 64;
             if (elect_one()) {
               if (h == 0 || k0 + 2 < kb_n) {
 #pragma unroll
@@ -672,7 +662,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
       const int row0 = t.m * a.tile_tok;
       const int rows = min(a.tile_tok, s_cnt[t.g] - row0);
       const uint32_t acc = jt & 1, aph = (jt >> 1) & 1;
-      if (!wait_warp(&tfull[acc], aph, abort_flag, lim)) break;
+      if (!mbar_wait_warp(&tfull[acc], aph, abort_flag, lim)) break;
       tc_fence_after();
       const uint32_t tb = tmem_base + ((uint32_t)(warp * 32) << 16) + acc * 128;
       const size_t orow = (size_t)(sh ? row0 : s_rb[t.g] + row0);
@@ -806,7 +796,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
         const CUtensorMap* map = sh ? &tmHS : &tmH;
         const int row = (sh ? 0 : s_rb[t.g]) + t.m * a.tile_tok;
         for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-          if (!wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+          if (!mbar_wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
           if (elect_one()) {
             if (tw < STEPS && k0 + tw < kb_n) {
               mbar_arrive_expect_tx(&sfull[r.i], n_it * 2048);
@@ -830,7 +820,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
         const int i2 = __shfl_sync(0xffffffffu, tok[0], q + 2), i3 = __shfl_sync(0xffffffffu, tok[0], q + 3);
         const uint32_t dst0 = smem_u32(sT) + w_stage + tw * 512 + lane * 2048, bar0 = smem_u32(sfull);
         for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-          if (!wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+          if (!mbar_wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
           const int ks = min(STEPS, kb_n - k0);
           if (elect_one()) {
             if (nq > 0) mbar_arrive_expect_tx(&sfull[r.i], ks * nq * 512);
@@ -855,7 +845,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
         }
         const uint32_t dst0 = smem_u32(sT) + w_stage + r0 * 128 + ((chunk ^ (r0 & 7)) << 4);
         for (int k0 = 0; k0 < kb_n; k0 += STEPS) {
-          if (!wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
+          if (!mbar_wait_warp(&sempty[r.i], r.ph ^ 1, abort_flag, lim)) { ok = false; break; }
           const uint32_t dst = dst0 + r.i * stage;
 #pragma unroll
           for (int i = 0; i < kRows; ++i) {
@@ -895,7 +885,7 @@ __global__ void __launch_bounds__(CCfg<Q4, STEPS, GATHER>::kThreads, 1)
     op.half = conv.half;
     op.sw = smem_u32(sW);
     op.ss = smem_u32(sS);
-    op.dst = tmem_base + ((uint32_t)(q * 32) << 16) + C::kOperandCol + set * 64;
+    op.dst = tmem_base + ((uint32_t)(q * 32) << 16) + kCOperandCol + set * 64;
     // the thread's row in a slot: down tiles in order, up tiles 64 gate rows,
     // then 64 up rows; 16-byte chunk c of row r lies at chunk c ^ (r & 7)
     const int at_dn = q * 32 + lane, at_up = (lane >> 4) * 64 + q * 16 + (lane & 15);
@@ -939,7 +929,7 @@ cudaError_t launch_cols(const CUtensorMap& tmW13, const CUtensorMap& tmW2, const
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(CCfg<Q4, STEPS, GATHER>::kThreads, 1, 1);
+  cfg.blockDim = dim3(cols_threads(Q4), 1, 1);
   cfg.dynamicSmemBytes = kColsFixed + a.ring_s * STEPS * ((Q4 ? 0 : kCSlot) + a.b_rows * 128) + a.ring_w * (kCSlot + kCScale);
   cfg.stream = s;
   cfg.attrs = attr;

@@ -194,7 +194,7 @@ struct FusedArgs {
   int tile_tok;                   // tokens per tile (32, 64 or 128)
   int steps;                      // 64-K steps per stage (2 or 4)
   int b_rows;                     // token rows per step in a stage (16 .. 128)
-  int ring_s, ring_w;             // stages; 4-bit: code slots (both powers of two)
+  int ring_s, ring_w;             // stages; 4-bit: code slots (there both are powers of two)
 };
 
 // ---------------------------------------------------------------------------
@@ -665,7 +665,8 @@ __device__ __forceinline__ uint32_t uniform(uint32_t v) {
   asm volatile("redux.sync.max.u32 %0, %1, 0xffffffff;" : "=r"(r) : "r"(v));
   return r;
 }
-// A wait of the whole warp, with one answer.
+// A wait of the whole warp, with one answer; the warp is converged after it
+// (what follows may be warp-wide or an aligned TMEM access).
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                long long limit) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit));

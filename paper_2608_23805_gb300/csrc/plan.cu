@@ -332,12 +332,11 @@ namespace {
 // of 16) and selects k + 1 <= 32 experts a token, one per lane of a warp.
 // Small layers (E <= 64 and E * H <= 32,768) take the FFMA router instead:
 // sized for 64 experts, its blocks finish in a few microseconds, below the
-// fixed cost of the tensor path's three launches (decode sizes).
+// fixed cost of the tensor path's two launches (decode sizes).
 bool tensor_router(const msi_plan_desc& d) {
   const int E = d.n_experts;
   if (E <= 64 && (long long)E * d.hidden <= 32768) return false;
-  return E % 16 == 0 && (E <= 128 || E % 128 == 0) && d.top_k <= 31 &&
-         E / std::min(E, 128) * std::min(d.top_k + 1, std::min(E, 128)) <= 160;
+  return E % 16 == 0 && (E <= 128 || E % 128 == 0) && d.top_k <= 31;
 }
 
 // A call that enqueues work must be made with the plan's device current: its
@@ -374,8 +373,11 @@ WsLayout layout(const msi_plan* p, int T) {
   L.total = take(12);     // 128-row tiles, 256-row pair tiles; the router selection's ticket
   L.sh_group = take(sizeof(Group));
   L.sh_total = take(8);
-  // the tensor router's logits (a longer call's go to the GEMMs' buffers, or
-  // through here in row chunks): at least 1.5 H rows
+  // the tensor router's logits, 4 E bytes a row: room for at least 1.5 H rows
+  // (a longer call's go to the GEMMs' buffers, or through here in row chunks).
+  // The size, 6 H bytes an expert and 8 bytes for each of a row's k + 1 per 128
+  // experts, decides with the rest which calls fit a given workspace (the
+  // static scratch above all), so it stays what callers have measured theirs by
   if (tensor_router(p->d)) {
     L.logits_bytes = 3 * E * H * 2 + 8 * (size_t)T * std::max<size_t>(1, E / 128) * std::min<size_t>(k + 1, E);
     L.logits = take(L.logits_bytes);

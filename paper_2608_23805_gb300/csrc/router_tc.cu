@@ -26,10 +26,11 @@
 //     the latency of one CTA's pass over K for short ones (one token: 24 us as
 //     4 CTAs of 128 experts, 16 as 32 of 16).  So short calls are cut into
 //     smaller expert chunks (router_chunk).
-//  2. router_select_kernel, one warp per token: selects the top k + 1, weights, gap, the 32-token block's expert histogram and the
-//     shared-expert gate sigmoid(x . w_sg).  A call of at most kFuseTokens
-//     tokens also does the scatter's work here (offsets, permutation,
-//     generation re-check, GEMM groups), in the CTA that finishes last.
+//  2. router_select_kernel, one warp per token: the top k + 1, weights, gap,
+//     the 32-token block's expert histogram and the shared-expert gate
+//     sigmoid(x . w_sg).  A call of at most kFuseTokens tokens also does the
+//     scatter's work here (offsets, permutation, generation re-check, GEMM
+//     groups), in the CTA that finishes last.
 #include "permute.cuh"
 
 namespace msi {
