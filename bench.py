@@ -70,13 +70,13 @@ L2_BYTES = 129 * 1024 * 1024
 # only while the GEMM source still hashes to the value the capture was taken at.
 TRAFFIC = {
     # one fused wave launch (gate-up + down of 32 experts, ~20,480 routed rows)
-    ("prefill32k_lru64", "gateup+down"): {"bytes_per_launch": 293416704 + 58600960, "src_hash": "60c33189754c4ab3",
+    ("prefill32k_lru64", "gateup+down"): {"bytes_per_launch": 293780480 + 59278848, "src_hash": "8b97b4cd0e07acda",
                                           "profile": "profiles/gemm_fused_wave_prefill32k_lru64.md"},
     # the fused launch of a 4K resident call
-    ("qwen3next_4k", "gateup+down"): {"bytes_per_launch": 3388616704 + 197220608, "src_hash": "60c33189754c4ab3",
+    ("qwen3next_4k", "gateup+down"): {"bytes_per_launch": 3386839040 + 196978688, "src_hash": "8b97b4cd0e07acda",
                                       "profile": "profiles/gemm_fused_qwen3next_4k.md"},
     # one fused 4-bit wave launch
-    ("prefill32k_q4_lru64", "gateup+down"): {"bytes_per_launch": 143731968 + 54402048, "src_hash": "60c33189754c4ab3",
+    ("prefill32k_q4_lru64", "gateup+down"): {"bytes_per_launch": 143790592 + 54549760, "src_hash": "8b97b4cd0e07acda",
                                              "profile": "profiles/gemm_fused_wave_q4_prefill32k_q4_lru64.md"},
 }
 

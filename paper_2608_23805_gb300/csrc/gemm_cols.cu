@@ -30,7 +30,8 @@
 //       traffic, which bounds the row-major 4-bit kernel.
 // Tokens (operand B), in the 128-byte swizzle, the tile's rows only: h by TMA in
 // boxes of 16 rows; x through the permutation, by TMA gathers of four rows up to
-// 64 tokens a tile, else by cp.async.  Copies and gathers by size (a call, us):
+// 64 tokens a tile, else by cp.async.  Copies and gathers by size (a call with the
+// shared expert in the launch, us):
 //   tokens               37    250    800   1,600   4,096
 //   cp.async, x and h   195    346    382     421     537
 //   gathers for x       187    334    369     427     562
@@ -41,9 +42,10 @@
 // What bounds it: for 4-bit the instructions of the converting and the issuing
 // warps (an MMA of up to 96 columns takes 48 cycles), not HBM; for bf16 and few
 // tokens the latency of a tile's pass over K.  Resident Qwen-shaped layer, both
-// projections: 4-bit 250 tokens 288 us (534 as two row-major launches), 8
-// tokens 62 us (91), 4,096 tokens 416 us (546); bf16 one token 24 us with the
-// shared expert (28 without it, which took 25 beside it).
+// projections: 4-bit 250 tokens 271 us (534 as two row-major launches), 4,096
+// tokens 393 us (546), 8 tokens 62 us with the shared expert (91 without it);
+// bf16 one token 26 us with the shared expert (row-major 28 without it, which
+// took 25 beside it).
 //
 // Schedule: every CTA takes a contiguous range of the up tiles, then of the
 // down tiles (ColsWalk), so a role steps from tile to tile without a search.

@@ -743,10 +743,11 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 }
 
 // Weights as MMA rows (gemm_cols.cu) while the groups average few rows:
-//   4-bit: at 8, 250 and 4,096 tokens of the Qwen-shaped layer 62, 288 and 416
-//     us against 91, 534 and 546 in two row-major launches; the call at 8,192
-//     tokens 964 against 1,209, at 20,000 (390 rows a group, four tiles and
-//     conversions) 2,105 against 2,215, at 32,768 3,508 against 3,086 on pairs.
+//   4-bit: at 250 and 4,096 tokens of the Qwen-shaped layer 271 and 393 us
+//     against 534 and 546 in two row-major launches; the call at 8,192 tokens
+//     912 against 1,209, at 20,000 (390 rows a group, four tiles and
+//     conversions) 2,104 against 2,235, at 25,000 2,628 against 2,681, at 32,768
+//     3,508 against 3,086 on pairs.
 //     64 experts, H 1,024, I 512, top_k 2: 4,000 to 14,000 rows 111 to 233
 //     against 120 to 244.  Small experts (few K steps and little to convert a
 //     tile, so that its hand-overs count) up to 24 rows a group: the call at 8,
@@ -756,7 +757,7 @@ msi_status validate_fwd(msi_plan* p, int layer, const void* x, int T, const floa
 //     A wave up to 256 rows (streamed calls of small experts, H 512, I 256: 16,
 //     62 and 125 rows a group 173, 200 and 209 against 208, 215 and 223).
 //   bf16: where the launches' latency is what counts, up to 256 rows with a
-//     shared expert, which this launch takes in (one token: 24 us for what took
+//     shared expert, which this launch takes in (one token: 26 us for what took
 //     28 + 25 on a side stream).  Calls, us, row-major and here, top_k 10 of 512
 //     experts: 37 rows 294 and 290, 200 rows 513 and 513, 400 rows 532 and 538;
 //     top_k 1 of 256: 250 rows 198 and 196, 1,000 rows 297 and 310, 2,000 rows
