@@ -160,7 +160,7 @@ struct FusedArgs {
   const __nv_bfloat16* x;   // [T, H]
   int x_ld;
   const int* perm;          // permuted row -> token
-  int* ready;               // [m-tiles] finished gate-up tiles per 128-row tile (zero at launch)
+  int* ready;               // finished gate-up tiles per 128-row tile (gemm_cols.cu: per token tile), zero at launch
   int* status;
   long long wait_limit;
   int stall;                // as GemmArgs::stall
